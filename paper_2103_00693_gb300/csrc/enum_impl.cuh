@@ -98,6 +98,57 @@ __device__ __forceinline__ void seed(const Table<W>& t, uint64_t i, uint64_t (&z
     }
 }
 
+// Seeds by table lookup. z(i) is linear in the bits of g(i), so 16 tables of
+// the combinations of four rows each give it in one lookup and one row XOR per
+// four bits, where seed() walks the set bits one by one (a chain of about 30
+// dependent shared-memory reads for a 60-bit index). z0 is folded into the
+// first table. An entry of one word per table: the 16 entries of a table lie in
+// 16 distinct bank pairs, so lanes with different indices read without
+// conflicts.
+constexpr int kSeedTables = 16;
+
+template <int W>
+struct SeedTable {
+    uint64_t t[W][kSeedTables][16];
+};
+
+// Tables covering the index bits that [0, last] uses.
+__host__ __device__ inline int seed_tables_for(uint64_t last)
+{
+    int bits = 1;
+    while (bits < 64 && (last >> bits)) ++bits;
+    return (bits + 3) / 4;
+}
+
+// Built by the whole CTA from a loaded table; the caller synchronises after.
+template <int W>
+__device__ __forceinline__ void build_seed_table(SeedTable<W>& st, const Table<W>& t, int ntab)
+{
+    for (int e = threadIdx.x; e < W * ntab * 16; e += blockDim.x) {
+        const int x = e & 15;
+        const int q = (e >> 4) % ntab;
+        const int w = (e >> 4) / ntab;
+        uint64_t v = q == 0 ? t.z0[w] : 0ull;
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+            if ((x >> b) & 1) v ^= t.B[4 * q + b][w];
+        st.t[w][q][x] = v;
+    }
+}
+
+template <int W>
+__device__ __forceinline__ void seed_lookup(const SeedTable<W>& st, int ntab, uint64_t i, uint64_t (&z)[W])
+{
+    uint64_t g = i ^ (i >> 1);
+#pragma unroll
+    for (int w = 0; w < W; ++w) z[w] = st.t[w][0][g & 15];
+    for (int q = 1; q < ntab; ++q) {
+        g >>= 4;
+#pragma unroll
+        for (int w = 0; w < W; ++w) z[w] ^= st.t[w][q][g & 15];
+    }
+}
+
 // Per-thread accumulator of the reduce, fed with solutions whose word 0 is in
 // the L domain (see load_table_hash_domain): sum of hashes and XOR-fold.
 template <int W>
@@ -159,19 +210,18 @@ struct GrayBlock<W, 0, Rows, Sink> {
     static __device__ __forceinline__ void run(uint64_t (&z)[W], const Rows&, Sink& sink) { sink.consume(z); }
 };
 
-// The reduce of [i, i + len). The solutions of an aligned block of 2^U
+// The reduce of [i, i + len), len >= 1, with z = z(i) (word 0 in the L domain).
+// The solutions of an aligned block of 2^U
 // consecutive indices (U >= 2) are z_s ^ XOR_{k in S} B_k over all subsets S
 // of {0..U-1}: z_s and every B_k occur an even number of times, so their
 // XOR is zero (in the L domain too, L being linear). Whole blocks therefore
 // feed only the hash; the head and the tail of the run (partial blocks) feed
 // hash and fold. The fold is exact, and one 64-bit XOR per solution lighter.
 template <int W, int U>
-__device__ __forceinline__ void reduce_run(const Table<W>& t, uint64_t i, uint64_t len, Acc<W>& acc)
+__device__ __forceinline__ void reduce_run_from(const Table<W>& t, uint64_t i, uint64_t len, uint64_t (&z)[W],
+                                                Acc<W>& acc)
 {
     static_assert(U >= 2, "a block of 2^U solutions XORs to zero only for U >= 2");
-    if (len == 0) return;
-    uint64_t z[W];
-    seed<W>(t, i, z);
     constexpr uint64_t kBlk = 1ull << U;
     while (len && (i & (kBlk - 1))) {  // head up to a multiple of 2^U
         acc.consume(z);
@@ -206,6 +256,15 @@ __device__ __forceinline__ void reduce_run(const Table<W>& t, uint64_t i, uint64
         ++i;
         if (len) xor_row<W>(z, t.B[ctz64(i)]);
     }
+}
+
+template <int W, int U>
+__device__ __forceinline__ void reduce_run(const Table<W>& t, uint64_t i, uint64_t len, Acc<W>& acc)
+{
+    if (len == 0) return;
+    uint64_t z[W];
+    seed<W>(t, i, z);
+    reduce_run_from<W, U>(t, i, len, z, acc);
 }
 
 // Block-wide (count, hsum, fold) reduction over a CTA of THREADS threads;

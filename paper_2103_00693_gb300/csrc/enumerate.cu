@@ -14,9 +14,12 @@
 //                        solutions are unrolled so that the first U basis
 //                        rows are compile-time register operands. The
 //                        per-thread (count, hash sum, XOR-fold) is reduced by
-//                        warp shuffles, shared memory and one 64-bit atomic
-//                        per quantity per CTA.
-//   reduce_chunks_kernel the same walk, one CTA per chunk, one result per chunk.
+//                        warp shuffles, shared memory and, where several
+//                        CTAs share a window, one 64-bit atomic per quantity
+//                        per CTA. One window or many (a result per chunk).
+//                        Windows too short to give a full wave long runs are
+//                        bound by how many threads walk them: runs go down
+//                        to one Gray block.
 //   store_kernel         coalesced materialisation. Lane t of a warp owns
 //                        index G*h + S*t (+1), G = 32*S. With m = log2 G,
 //                          g(G h + t) = (g(h) << m) ^ ((h & 1) << (m-1)) ^ g(t),
@@ -36,65 +39,57 @@ namespace {
 
 
 
+// The reduce of n_chunks windows of `chunk` indices, window c starting at
+// offset + c * chunk (hlf_enumerate_reduce is one window). A window is cut into
+// `parts` CTAs of blockDim.x threads, each thread walking `per` consecutive
+// indices that start at a multiple of 2^U, so that only the window's two ends
+// have partial Gray blocks. Items (window, part) are taken grid-stride. With
+// one part per window the CTA writes the result; otherwise it adds to it.
 template <int W, int U, int T>
-__global__ void __launch_bounds__(T, min_ctas_for(W)) reduce_kernel(const uint64_t* __restrict__ table,
-                                                                   uint64_t offset, uint64_t count,
-                                                                   uint64_t per_thread, uint64_t threads_used,
-                                                                   hlf_reduce* __restrict__ out)
+__global__ void __launch_bounds__(T, min_ctas_for(W))
+    reduce_kernel(const uint64_t* __restrict__ table, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
+                  uint32_t parts, uint64_t per, uint64_t runs, uint64_t align, int ntab,
+                  hlf_reduce* __restrict__ out)
 {
     __shared__ Table<W> t;
+    __shared__ SeedTable<W> st;
     load_table_hash_domain<W>(t, table);
     __syncthreads();
-    const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    Acc<W> acc;
-    acc.zero();
-    uint64_t cnt = 0;
-    if (g < threads_used) {
-        const uint64_t a = g * per_thread;
-        if (a < count) {
-            const uint64_t len = min(per_thread, count - a);
-            cnt = len;
-            reduce_run<W, U>(t, offset + a, len, acc);
-        }
-    }
-    block_reduce<W, T>(cnt, acc);
-    if (threadIdx.x == 0 && cnt) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(&out->count), (unsigned long long)cnt);
-        atomicAdd(reinterpret_cast<unsigned long long*>(&out->hsum), (unsigned long long)acc.hs);
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            const uint64_t f = acc.fold_word(w);
-            if (f) atomicXor(reinterpret_cast<unsigned long long*>(&out->xor_fold[w]), (unsigned long long)f);
-        }
-    }
-}
-
-template <int W, int U>
-__global__ void __launch_bounds__(kThreads) reduce_chunks_kernel(const uint64_t* __restrict__ table,
-                                                                 uint64_t offset, uint64_t chunk,
-                                                                 uint64_t n_chunks, hlf_reduce* __restrict__ out)
-{
-    __shared__ Table<W> t;
-    load_table_hash_domain<W>(t, table);
+    build_seed_table<W>(st, t, ntab);
     __syncthreads();
-    const uint64_t per_thread = (chunk + blockDim.x - 1) / blockDim.x;
-    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+    for (uint64_t item = blockIdx.x; item < n_chunks * parts; item += gridDim.x) {
+        const uint64_t c = item / parts;
+        const uint64_t first = offset + c * chunk;
+        const uint64_t skip = first & align;  // indices before the window in its first block
+        const uint64_t run = (item - c * parts) * blockDim.x + threadIdx.x;
+        const uint64_t a = run * per;  // counted from that block's start
         Acc<W> acc;
         acc.zero();
         uint64_t cnt = 0;
-        const uint64_t a = threadIdx.x * per_thread;
-        if (a < chunk) {
-            const uint64_t len = min(per_thread, chunk - a);
-            cnt = len;
-            reduce_run<W, U>(t, offset + c * chunk + a, len, acc);
+        const uint64_t lo = max(a, skip);
+        if (run < runs && lo - skip < chunk) {
+            cnt = min(per - (lo - a), chunk - (lo - skip));
+            uint64_t z[W];
+            const uint64_t i = first + (lo - skip);
+            seed_lookup<W>(st, ntab, i, z);
+            reduce_run_from<W, U>(t, i, cnt, z, acc);
         }
-        block_reduce<W>(cnt, acc);
-        if (threadIdx.x == 0) {
-            hlf_reduce& r = out[c];
+        block_reduce<W, T>(cnt, acc);
+        if (threadIdx.x != 0) continue;
+        hlf_reduce& r = out[c];
+        if (parts == 1) {
             r.count = cnt;
             r.hsum = acc.hs;
 #pragma unroll
-            for (int w = 0; w < HLF_MAX_W; ++w) r.xor_fold[w] = w < W ? acc.fold_word(w) : 0ull;
+            for (int w = 0; w < HLF_MAX_W; ++w) r.xor_fold[w] = w < W ? acc.fold_word(w < W ? w : 0) : 0ull;
+        } else if (cnt) {
+            atomicAdd(reinterpret_cast<unsigned long long*>(&r.count), (unsigned long long)cnt);
+            atomicAdd(reinterpret_cast<unsigned long long*>(&r.hsum), (unsigned long long)acc.hs);
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                const uint64_t f = acc.fold_word(w);
+                if (f) atomicXor(reinterpret_cast<unsigned long long*>(&r.xor_fold[w]), (unsigned long long)f);
+            }
         }
     }
 }
@@ -215,42 +210,97 @@ int blocks_per_sm(K kernel, size_t smem)
     return fit;
 }
 
-template <int W>
-hlf_status launch_reduce_w(const uint64_t* table, uint64_t offset, uint64_t count, hlf_reduce* out,
-                           cudaStream_t s)
+// How a reduce of n_chunks windows of `chunk` indices is cut: CTAs of
+// `threads`, `parts` of them per window, `per` indices per thread.
+struct ReduceShape {
+    unsigned threads, blocks;
+    uint32_t parts;
+    uint64_t per, runs;
+    uint64_t align;  // runs start at multiples of align + 1
+};
+
+// The threads a window can use are one per Gray block of 2^U indices; a seed
+// costs a few tens of solutions (kSeedCost), so short runs are worth it
+// whenever they fill idle SMs. One window: one CTA if that holds them all (the
+// result then needs no clearing), else all of them, up to one wave, in CTAs no
+// larger than spreading them over every SM takes. Several windows: the largest
+// CTA a window fills, and the cut whose waves cost least.
+// With runs of at least 2048 indices and one CTA per window instead, 2^20
+// four-word solutions took 694 us on one SM (now 12.4, two launches and the
+// host's call among it), and 64 windows of 2^24 at W = 1 took 2.16 ms on 64
+// CTAs of 256 threads (now 0.79).
+template <int W, int U, int T>
+ReduceShape reduce_shape(uint64_t chunk, uint64_t n_chunks)
 {
-    constexpr int U = reduce_unroll(W);
+    constexpr uint64_t kSeedCost = 48;
+    const uint64_t sms = (uint64_t)sm_count();
+    const uint64_t runs = ((chunk - 1) >> U) + 2;  // Gray blocks the window touches, at most
+    const uint64_t room = (uint64_t)min_ctas_for(W) * T;  // threads an SM holds
+    ReduceShape sh{};
+    uint64_t want;  // threads for the window
+    if (n_chunks == 1) {
+        want = runs < sms * room ? runs : sms * room;
+        uint64_t bd = want <= T ? want : (want + sms - 1) / sms;
+        bd = (bd + 31) / 32 * 32;
+        bd = bd > T ? T : (want > T && bd < 128 ? 128 : bd);
+        sh.threads = (unsigned)bd;
+        sh.parts = (uint32_t)((want + bd - 1) / bd);
+    } else {
+        uint64_t bd = T;
+        while (bd > 64 && bd > runs) bd /= 2;
+        sh.threads = (unsigned)bd;
+        const uint64_t slots = sms * (room / bd);
+        uint64_t best = ~0ull;
+        for (uint64_t k = 1; k <= 64 && (k == 1 || (k - 1) * bd < runs); ++k) {
+            const uint64_t waves = (n_chunks * k + slots - 1) / slots;
+            const uint64_t cost = waves * (kSeedCost + (chunk + k * bd - 1) / (k * bd));
+            if (cost < best) {
+                best = cost;
+                sh.parts = (uint32_t)k;
+            }
+            if (n_chunks > (~0ull >> 8)) break;  // a window each is enough
+        }
+    }
+    want = (uint64_t)sh.parts * sh.threads;
+    // chunk + 2^U - 1 indices at most, counted from the window's first block;
+    // past 2^63 that count could wrap, so such windows start their runs at the
+    // window's own start
+    sh.align = chunk <= 1ull << 63 ? (1ull << U) - 1 : 0;
+    sh.per = chunk / want + (chunk % want + sh.align + want - 1) / want;
+    sh.per = (sh.per + (1ull << U) - 1) & ~((1ull << U) - 1);
+    sh.runs = sh.align ? want : (chunk - 1) / sh.per + 1;
+    const uint64_t items = n_chunks * sh.parts;
+    const uint64_t cap = sms * (room / sh.threads);
+    sh.blocks = (unsigned)(items < cap ? items : cap);
+    return sh;
+}
+
+template <int W, int U>
+hlf_status launch_reduce_u(const uint64_t* table, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
+                           hlf_reduce* out, cudaStream_t s)
+{
     constexpr int T = reduce_threads(W);
-    // one wave: as many CTAs as fit on every SM at once
-    static int fit[64] = {0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 64 && fit[dev] == 0 &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit[dev], reduce_kernel<W, U, T>, T, 0) != cudaSuccess)
+    const ReduceShape sh = reduce_shape<W, U, T>(chunk, n_chunks);
+    if (sh.parts > 1 && cudaMemsetAsync(out, 0, sizeof(hlf_reduce) * n_chunks, s) != cudaSuccess)
         return HLF_ERR_CUDA;
-    const int per_sm = (dev < 64 && fit[dev] > 0) ? fit[dev] : 1;
-    const uint64_t max_threads = (uint64_t)sm_count() * per_sm * T;
-    const uint64_t min_run = 2048;  // amortises the <= 64-row seed
-    uint64_t threads = (count + min_run - 1) / min_run;
-    if (threads > max_threads) threads = max_threads;
-    if (threads == 0) threads = 1;
-    uint64_t per_thread = (count + threads - 1) / threads;
-    per_thread = (per_thread + (1ull << U) - 1) & ~((1ull << U) - 1);  // keep runs aligned
-    const uint64_t used = (count + per_thread - 1) / per_thread;
-    const unsigned blocks = (unsigned)((used + T - 1) / T);
-    reduce_kernel<W, U, T><<<blocks, T, 0, s>>>(table, offset, count, per_thread, used, out);
+    const int ntab = seed_tables_for(offset + (chunk * n_chunks - 1));
+    reduce_kernel<W, U, T><<<sh.blocks, sh.threads, 0, s>>>(table, offset, chunk, n_chunks, sh.parts, sh.per, sh.runs,
+                                                           sh.align, ntab, out);
     return cudaGetLastError() == cudaSuccess ? HLF_OK : HLF_ERR_CUDA;
 }
 
+// W = 1 has two unrolls: 2^6 solutions per Gray block where every thread of a
+// full wave has at least 16 blocks, else 2^3, whose finer cut balances and
+// fills the SMs better than the deeper unroll saves.
 template <int W>
-hlf_status launch_reduce_chunks_w(const uint64_t* table, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
-                                  hlf_reduce* out, cudaStream_t s)
+hlf_status launch_reduce_w(const uint64_t* table, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
+                           hlf_reduce* out, cudaStream_t s)
 {
-    constexpr int U = reduce_unroll(W);
-    const uint64_t cap = (uint64_t)sm_count() * blocks_per_sm(reduce_chunks_kernel<W, U>, 0);
-    const unsigned blocks = (unsigned)(n_chunks < cap ? n_chunks : cap);
-    reduce_chunks_kernel<W, U><<<blocks, kThreads, 0, s>>>(table, offset, chunk, n_chunks, out);
-    return cudaGetLastError() == cudaSuccess ? HLF_OK : HLF_ERR_CUDA;
+    if constexpr (W == 1) {
+        const uint64_t wave = (uint64_t)sm_count() * min_ctas_for(1) * reduce_threads(1);
+        if (chunk * n_chunks < wave * 1024) return launch_reduce_u<1, 3>(table, offset, chunk, n_chunks, out, s);
+    }
+    return launch_reduce_u<W, reduce_unroll(W)>(table, offset, chunk, n_chunks, out, s);
 }
 
 template <int W>
@@ -344,18 +394,10 @@ hlf_status launch_sample_w(const uint64_t* table, int nb, const uint64_t* idx, u
 
 }  // namespace
 
-hlf_status launch_reduce(const uint64_t* table, int W, uint64_t offset, uint64_t count, hlf_reduce* out,
-                         cudaStream_t s)
+hlf_status launch_reduce(const uint64_t* table, int W, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
+                         hlf_reduce* out, cudaStream_t s)
 {
-#define CALL(w) launch_reduce_w<w>(table, offset, count, out, s)
-    HLF_DISPATCH_W(W, CALL)
-#undef CALL
-}
-
-hlf_status launch_reduce_chunks(const uint64_t* table, int W, uint64_t offset, uint64_t chunk,
-                                uint64_t n_chunks, hlf_reduce* out, cudaStream_t s)
-{
-#define CALL(w) launch_reduce_chunks_w<w>(table, offset, chunk, n_chunks, out, s)
+#define CALL(w) launch_reduce_w<w>(table, offset, chunk, n_chunks, out, s)
     HLF_DISPATCH_W(W, CALL)
 #undef CALL
 }

@@ -539,9 +539,11 @@ hlf_status hlf_enumerate_reduce(hlf_handle* h, uint64_t offset, uint64_t count, 
     if (st != HLF_OK) return st;
     if (!window_ok(h->r, offset, count)) return HLF_ERR_RANGE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(red_dev, 0, sizeof(hlf_reduce), s) != cudaSuccess) return HLF_ERR_CUDA;
-    if (count == 0) return after_launch(h, HLF_OK, s);
-    return after_launch(h, hlf::launch_reduce(enum_table(h), h->W, offset, count, red_dev, s), s);
+    if (count == 0) {
+        if (cudaMemsetAsync(red_dev, 0, sizeof(hlf_reduce), s) != cudaSuccess) return HLF_ERR_CUDA;
+        return after_launch(h, HLF_OK, s);
+    }
+    return after_launch(h, hlf::launch_reduce(enum_table(h), h->W, offset, count, 1, red_dev, s), s);
 }
 
 hlf_status hlf_enumerate_histogram(hlf_handle* h, uint64_t offset, uint64_t count, int32_t bit_lo, int32_t nbits,
@@ -575,7 +577,7 @@ hlf_status hlf_enumerate_reduce_chunks(hlf_handle* h, uint64_t offset, uint64_t 
     if (!window_ok(h->r, offset, chunk * n_chunks)) return HLF_ERR_RANGE;
     if (n_chunks == 0) return HLF_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    return after_launch(h, hlf::launch_reduce_chunks(enum_table(h), h->W, offset, chunk, n_chunks, red_dev, s), s);
+    return after_launch(h, hlf::launch_reduce(enum_table(h), h->W, offset, chunk, n_chunks, red_dev, s), s);
 }
 
 hlf_status hlf_sample(hlf_handle* h, const uint64_t* idx_dev, uint64_t m, uint64_t* out_dev, void* stream)

@@ -110,10 +110,10 @@ constexpr int kFactorWorkWords = 64;
 
 // ---------------------------------------------------------------- launchers
 hlf_status launch_factor(const uint64_t* A, int n, int W, const FactorOut& o, cudaStream_t s);
-hlf_status launch_reduce(const uint64_t* table, int W, uint64_t offset, uint64_t count,
+// The reduce of n_chunks windows of `chunk` >= 1 indices each, one result per
+// window, all of it overwritten.
+hlf_status launch_reduce(const uint64_t* table, int W, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
                          hlf_reduce* out, cudaStream_t s);
-hlf_status launch_reduce_chunks(const uint64_t* table, int W, uint64_t offset, uint64_t chunk,
-                                uint64_t n_chunks, hlf_reduce* out, cudaStream_t s);
 // out: 8-byte aligned at W = 1, 16-byte aligned at W > 1.
 hlf_status launch_store(const uint64_t* table, int W, uint64_t offset, uint64_t count,
                         uint64_t* out, cudaStream_t s);
