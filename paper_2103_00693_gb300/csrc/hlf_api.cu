@@ -558,8 +558,10 @@ hlf_status hlf_enumerate_histogram(hlf_handle* h, uint64_t offset, uint64_t coun
     if (st != HLF_OK) return st;
     if (!window_ok(h->r, offset, count)) return HLF_ERR_RANGE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(hist_dev, 0, sizeof(uint64_t) << nbits, s) != cudaSuccess) return HLF_ERR_CUDA;
-    if (count == 0) return after_launch(h, HLF_OK, s);
+    if (count == 0) {
+        if (cudaMemsetAsync(hist_dev, 0, sizeof(uint64_t) << nbits, s) != cudaSuccess) return HLF_ERR_CUDA;
+        return after_launch(h, HLF_OK, s);
+    }
     return after_launch(h, hlf::launch_histogram(h->order == HLF_ORDER_PAPER ? h->ptable : h->table, h->W, offset,
                                                  count, bit_lo, nbits, hist_dev, s), s);
 }

@@ -49,7 +49,7 @@ enum DebugSite : int {
     kSiteDenseStore = 6, // dense kernels: stream words vs the stream's length
     kSiteFactorSmem = 7, // factor: panel tables, pivot lists, basis rows
     kSiteFactorKvec = 8, // factor_kvec_kernel: mask words, x_f words, table words
-    kSiteHistBin = 9,    // histogram kernels: bins vs the bin count
+    kSiteHistBin = 9,    // histogram kernel: bins vs the bin count
 };
 
 #ifdef HLF_DEBUG
@@ -119,6 +119,7 @@ hlf_status launch_store(const uint64_t* table, int W, uint64_t offset, uint64_t 
                         uint64_t* out, cudaStream_t s);
 hlf_status launch_store_dense(const uint64_t* table, int n, uint64_t offset, uint64_t count, uint64_t* out,
                               cudaStream_t s);
+// count >= 1; every bin is written.
 hlf_status launch_histogram(const uint64_t* table, int W, uint64_t offset, uint64_t count, int lo, int nbits,
                             uint64_t* out, cudaStream_t s);
 hlf_status launch_sample(const uint64_t* table, int W, int nb, const uint64_t* idx, uint64_t m,
