@@ -83,10 +83,7 @@ constexpr size_t batch_smem_bytes()
 {
     constexpr int NW = T / 32;
     size_t m = 0;
-    m = factor_smem_bytes<1, kBatchMaxN, NW>(kBatchMaxN) > m ? factor_smem_bytes<1, kBatchMaxN, NW>(kBatchMaxN) : m;
-    m = factor_smem_bytes<2, kBatchMaxN, NW>(kBatchMaxN) > m ? factor_smem_bytes<2, kBatchMaxN, NW>(kBatchMaxN) : m;
-    m = factor_smem_bytes<3, kBatchMaxN, NW>(kBatchMaxN) > m ? factor_smem_bytes<3, kBatchMaxN, NW>(kBatchMaxN) : m;
-    m = factor_smem_bytes<4, kBatchMaxN, NW>(kBatchMaxN) > m ? factor_smem_bytes<4, kBatchMaxN, NW>(kBatchMaxN) : m;
+    m = factor_smem_bytes<4, kBatchMaxN>(kBatchMaxN, true) > m ? factor_smem_bytes<4, kBatchMaxN>(kBatchMaxN, true) : m;
     // store chunks: table, step rows C_j, per-warp staging
     const size_t st = sizeof(Table<kBatchMaxW>) + sizeof(uint64_t) * (kTableRows - kStoreM) * kBatchMaxW +
                       sizeof(uint64_t) * NW * stage_words<kBatchMaxW>();
@@ -114,7 +111,8 @@ template <int W, int T>
 __device__ void batch_factor(const BatchArgs& a, int b, int n, const uint64_t* A, unsigned char* smem)
 {
     FactorOut o{nullptr, nullptr, a.tables + (size_t)b * kTableSlot, a.info + kInfo * b, nullptr};
-    factor_block<W, kBatchMaxN / T, kBatchMaxN, T / 32>(A, n, o, smem);
+    constexpr int rt = 32 * row_warps(T / 32);
+    factor_block<W, (64 * W + rt - 1) / rt, kBatchMaxN>(A, n, o, smem);
 }
 
 template <int W, int T>

@@ -1,33 +1,23 @@
-// Stage 1 of the two-stage scheme as a block-level device function: the CLA
+// Stage 1 of the two-stage scheme as block-level device functions: the CLA
 // module of Section 2 (Fig. 1(b)), steps (1)-(4), for one matrix per CTA.
 //
-//   (1) Gauss-Jordan elimination of A over GF(2). Each thread owns R rows of
-//       A in registers (W uint64 words each). For each column c, left to
-//       right, the candidates are the rows not yet used as a pivot that have
-//       bit c set; a min over each warp and then over the warps picks the
-//       lowest such row p. The key minimised is (row << 5) | warp, so the
-//       minimum also names the warp that holds row p. Each warp stages its
-//       lowest candidate's words next to its key, so one barrier per column
-//       suffices: after it every thread knows p and reads row p from that
-//       warp's slot, and every other row with bit c set XORs it in (rows
-//       above and below: Gauss-Jordan, so the result is the unique reduced
-//       row echelon form). The slots
-//       alternate with the column's parity, so a slot is rewritten only after
-//       the next column's barrier, when every read of it is done. A row not
-//       yet used as a pivot is zero in every column left of c (each earlier
-//       column was cleared by its pivot or had no candidate), so the pivot
-//       row's words left of c's word are zero: they are neither staged nor
-//       XORed. Rows are never swapped; the pivot row of column c is
-//       remembered instead. Unused rows end at zero.
-//
-//       Measured and rejected: one warp eliminating alone with ballots and
-//       shuffles (slower from W = 2 on), and two columns per barrier (three
-//       minima per warp; more work per column than the barrier it saves).
+//   (1) Gauss-Jordan elimination of A over GF(2). The reduced row echelon form
+//       is unique, so any row with the column's bit may be the pivot; nothing
+//       asks for the lowest one, and no exchange across the CTA is needed per
+//       column: one warp finds the pivots alone.
+//       W = 1 (eliminate_warp): the warp holds whole rows, two a lane, and
+//       the pivot row of column c moves to position c. A pivot is one warp
+//       maximum of the remaining words, with the columns from the top bit down.
+//       W > 1 (eliminate_panels): panels of 32 columns. One warp, which owns no
+//       rows, eliminates the 32-bit slices of the live rows (unused, slice not
+//       zero); the row warps then apply what it found to whole rows. See there.
 //   (2)-(4) Kernel basis, q and z^a. For a free column f the kernel vector is
 //       x_f = e_f + sum_k B_k[f] e_{p_k}; q(x_f) = sum over i in supp(x_f) of
 //       popcount(A_i & x_f), mod 4, which is x_f^T A x_f mod 4. With z^a
 //       chosen to vanish on the pivots, z^a . x_f = z^a_f, so the equation
-//       2 z^T x_f = q(x_f) (mod 4) gives z^a_f = q(x_f) / 2 directly.
+//       2 z^T x_f = q(x_f) (mod 4) gives z^a_f = q(x_f) / 2 directly. Bit p of
+//       x_f is bit f of the row whose pivot is p, so 32 bits of x_f are one
+//       ballot over 32 positions.
 //
 // Also checked here: padding bits (column >= n) are zero and A is symmetric
 // (Section 1 defines the problem for symmetric A only), the latter by 64 x 64
@@ -37,18 +27,6 @@
 #include "hlf_internal.cuh"
 
 namespace hlf {
-
-// NW: the most warps a CTA running factor_block may have (32 by default).
-template <int W, int MAXN, int NW = 32>
-struct FactorSmem {
-    int first[2][NW];        // per warp: its lowest candidate's key for the column (by column parity)
-    uint64_t crow[2][NW][W];  // and that row's words
-    int pivcol[MAXN];
-    uint32_t pivmask[MAXN / 32];
-    uint64_t x[NW][W];
-    uint64_t z0[W];
-    int err;
-};
 
 // Transpose a 64 x 64 bit block held by one warp: lane l has rows l (x0) and
 // l + 32 (x1), bit s of a row being column s. Stage j (j = 32, 16, ..., 1)
@@ -81,61 +59,483 @@ __device__ __forceinline__ void transpose64_warp(uint64_t& x0, uint64_t& x1, int
     }
 }
 
-// Row stride of the basis rows in shared memory: odd, so that 32 lanes reading
-// one word of 32 consecutive rows hit distinct banks.
-template <int W>
-constexpr int basis_stride() { return W | 1; }
+// ------------------------------------------------------------ elimination
 
-template <int W, int MAXN, int NW = 32>
-constexpr size_t factor_smem_bytes(int n)
+constexpr int kPanelCap = 128;  // slices the searching warp takes at most (4 a lane)
+
+// Slices a search takes when nl rows are live. Beyond the most that fit, 64: rows
+// as many as that nearly always span the panel, and a shorter column costs less;
+// where they do not, the panel is searched again for what the others still hold.
+__device__ __forceinline__ int panel_cap(int nl)
 {
-    return sizeof(FactorSmem<W, MAXN, NW>) + (size_t)n * basis_stride<W>() * sizeof(uint64_t);
+    return nl <= 32 ? 32 : (nl <= 64 || nl > kPanelCap ? 64 : kPanelCap);
 }
 
-// Factor the n x n matrix A ([n][W] words, global) with the whole CTA.
-// Thread t owns the R rows t, t + blockDim.x, ... in registers. Requires
-// R * blockDim.x >= n, blockDim.x a multiple of 32 and at most 32 * NW,
-// n <= MAXN. `smem` points to factor_smem_bytes<W, MAXN, NW>(n) bytes of
-// shared memory. Writes o.table
-// (always), o.basis and o.piv (when non-null) and o.info[0] = status,
-// o.info[1] = r (or -1 on a fault). Returns r, or -1.
-template <int W, int R, int MAXN, int NW = 32>
-__device__ int factor_block(const uint64_t* __restrict__ A, int n, const FactorOut& o, unsigned char* smem)
+// Whether no row can hold further pivots of the panel: none was live, all that
+// were have been searched, or every column has its pivot. (A live slice has a
+// bit, so a search of any finds at least one pivot and this ends.)
+__device__ __forceinline__ bool panel_done(int nl, uint32_t cols, int ncols)
 {
-    constexpr int kNone = 0x7fffffff;
-    using Smem = FactorSmem<W, MAXN, NW>;
+    return cols == 0u || nl <= panel_cap(nl) || __popc(cols) == ncols;
+}
+
+// Shared memory of a factorisation of up to MAXN rows of W words. The arrays
+// sized by n follow it: rows [W][stride] (word-major: a warp's rows are
+// consecutive; the stride is odd, so the words of one row lie in distinct banks
+// too) and T2 [8][W][16] (W > 1), and for factor_block a copy of A like rows.
+template <int W, int MAXN>
+struct FactorSmem {
+    uint32_t list[kPanelCap];    // slices of the live rows
+    int16_t listrow[kPanelCap];  // and the rows
+    int16_t kres[kPanelCap];     // the column each searched slice became the pivot of, or -1
+    __align__(8) int16_t prow[2][32];  // the pivot row of column b, -1 if free, by round parity
+    int nlist[2];              // live rows, by round parity
+    int nactive;               // rows that absorb pivots of the last panel
+    uint32_t cols;             // the search's pivot columns
+    __align__(16) uint32_t Hcol[32];  // reduced pivot row of column b as a set of pivot start rows, 0 if free
+    uint32_t T1[8 * 16];       // XORs of Hcol over 4 columns
+    int err;
+    int rank;
+    uint64_t z0[W];
+    uint32_t pivmask[MAXN / 32];  // the pivot columns, one bit each
+    int before[MAXN / 32];        // pivots in the mask words before
+    uint2 active[MAXN];           // (row, coefficient set)
+    int16_t rowof[MAXN];          // the row whose pivot is column c, -1 if c is free
+    int16_t pivcol[MAXN];         // p_k
+    int16_t rowk[MAXN];           // the row that holds B_k
+};
+
+template <int W>
+__host__ __device__ constexpr int row_stride(int n) { return W == 1 ? 64 : (n | 1); }
+
+template <int W, int MAXN>
+__host__ __device__ constexpr size_t factor_smem_bytes(int n, bool with_copy)
+{
+    return (sizeof(FactorSmem<W, MAXN>) + 15) / 16 * 16 +
+           sizeof(uint64_t) * W * ((size_t)row_stride<W>(n) * (with_copy ? 2 : 1) + (W > 1 ? 8 * 16 : 0));
+}
+
+template <int W, int MAXN>
+__device__ __forceinline__ uint64_t* factor_rows(unsigned char* smem)
+{
+    return reinterpret_cast<uint64_t*>(smem + (sizeof(FactorSmem<W, MAXN>) + 15) / 16 * 16);
+}
+
+// A value that is the same in every lane of the warp, in a form that lets the
+// compiler know it: a branch on it keeps the warp converged. Behind a branch that
+// might split the warp every warp-wide operation is preceded by a
+// reconvergence, which doubled the time of the searches below.
+__device__ __forceinline__ int warp_uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+// The warps of an elimination (W > 1). An SM's four schedulers take a CTA's warps
+// by their number mod 4. The searching warp is a serial chain of instructions, so
+// it has a scheduler to itself: it is warp 3, the row warps are those whose number
+// is not 3 mod 4, and the others stand idle until the elimination is done. Next to
+// row warps on its scheduler the search of a panel took up to twice as long (n =
+// 1024). A CTA of fewer than four warps has its last warp search.
+__host__ __device__ constexpr int search_warp(int nwarps) { return nwarps >= 4 ? 3 : nwarps - 1; }
+__host__ __device__ constexpr int row_warps(int nwarps) { return nwarps >= 4 ? nwarps - nwarps / 4 : nwarps - 1; }
+// The threads of a CTA with at least `want` row threads.
+__host__ __device__ constexpr int elim_threads(int want)
+{
+    const int rw = (want + 31) / 32;
+    const int last = rw - 1 + (rw - 1) / 3;  // the last row warp's number
+    return 32 * (last + 1 < 4 ? 4 : last + 1);
+}
+
+// A barrier of the row warps and the searching warp, reached from different code.
+__device__ __forceinline__ void bar_elim(int rt)
+{
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"r"(rt + 32) : "memory");
+}
+
+// W = 1: one warp, the CTA's first, eliminates the whole matrix. Lane
+// l's candidates are rows l and l + 32, columns 0..31 and 32..63 in a word each,
+// bit-reversed so that the leftmost column is the top bit. The largest left word
+// of all candidates has the column's bit if any has, so one warp maximum both
+// tells whether the column has a pivot and broadcasts the pivot row's word; the
+// right word is a second maximum over the rows that share the left one (any of
+// them may be the pivot). The pivot row XORs itself to zero where it was and
+// lives on at its column's position (lane c & 31), where later pivots clear their
+// columns. No step branches: without a pivot no candidate has the bit.
+template <int MAXN>
+__device__ void eliminate_warp(const uint64_t* __restrict__ A, int n, unsigned char* smem, uint64_t* copy)
+{
+    using Smem = FactorSmem<1, MAXN>;
     Smem& sm = *reinterpret_cast<Smem*>(smem);
-    constexpr int SW = basis_stride<W>();
-    uint64_t* s_rows = reinterpret_cast<uint64_t*>(smem + sizeof(Smem));  // [n][SW]
-
-    const int tid = threadIdx.x;
-    const int bs = blockDim.x;
-    const int lane = tid & 31;
-    const int warp = tid >> 5;
-    const int nwarps = bs >> 5;
-
-    uint64_t row[R][W];
+    uint64_t* s_rows = factor_rows<1, MAXN>(smem);  // by pivot column
+    const int lane = threadIdx.x;
+    uint64_t a0 = lane < n ? A[lane] : 0ull;
+    uint64_t a1 = lane + 32 < n ? A[lane + 32] : 0ull;
+    copy[lane] = a0;
+    copy[lane + 32] = a1;
+    a0 = __brevll(a0);
+    a1 = __brevll(a1);
+    uint32_t r0a = (uint32_t)(a0 >> 32), r0b = (uint32_t)a0, r1a = (uint32_t)(a1 >> 32), r1b = (uint32_t)a1;
+    uint32_t z0a = 0, z0b = 0, z1b = 0;  // positions lane and lane + 32 (whose left words stay zero)
+    uint32_t q = __reduce_max_sync(0xffffffffu, max(r0a, r1a));
 #pragma unroll
-    for (int j = 0; j < R; ++j) {
-        const int i = tid + j * bs;
-#pragma unroll
-        for (int w = 0; w < W; ++w) row[j][w] = i < n ? A[(size_t)i * W + w] : 0ull;
+    for (int c = 0; c < 32; ++c) {
+        if (c % 8 == 0 && !q) break;
+        const uint32_t L = 0x80000000u >> c;
+        const bool piv = q & L;
+        const uint32_t qb =
+            __reduce_max_sync(0xffffffffu, max(r0a == q ? r0b : 0u, r1a == q ? r1b : 0u));
+        const uint32_t qa = q;
+        const bool h0 = r0a & L, h1 = r1a & L, hz = piv && (z0a & L);
+        r0a ^= h0 ? qa : 0u;
+        r1a ^= h1 ? qa : 0u;
+        q = __reduce_max_sync(0xffffffffu, max(r0a, r1a));
+        r0b ^= h0 ? qb : 0u;
+        r1b ^= h1 ? qb : 0u;
+        z0a ^= hz ? qa : 0u;
+        z0b ^= hz ? qb : 0u;
+        if (piv && lane == c) {
+            z0a = qa;
+            z0b = qb;
+        }
     }
-    if (tid == 0) sm.err = 0;
-    if (tid < W) sm.z0[tid] = 0;
-    for (int i = tid; i < MAXN / 32; i += bs) sm.pivmask[i] = 0;
+    q = __reduce_max_sync(0xffffffffu, max(r0b, r1b));
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+        if (c % 8 == 0 && !q) break;
+        const uint32_t L = 0x80000000u >> c;
+        const bool piv = q & L;
+        const uint32_t qb = q;
+        r0b ^= r0b & L ? qb : 0u;
+        r1b ^= r1b & L ? qb : 0u;
+        q = __reduce_max_sync(0xffffffffu, max(r0b, r1b));
+        z0b ^= piv && (z0b & L) ? qb : 0u;
+        z1b ^= piv && (z1b & L) ? qb : 0u;
+        if (piv && lane == c) z1b = qb;
+    }
+    s_rows[lane] = __brevll(((uint64_t)z0a << 32) | z0b);
+    s_rows[lane + 32] = __brevll((uint64_t)z1b);
+    const unsigned m0 = __ballot_sync(0xffffffffu, z0a != 0u), m1 = __ballot_sync(0xffffffffu, z1b != 0u);
+    if (lane == 0) {
+        sm.pivmask[0] = m0;
+        sm.pivmask[1] = m1;
+    }
+    sm.rowof[lane] = z0a ? (int16_t)lane : (int16_t)-1;
+    sm.rowof[lane + 32] = z1b ? (int16_t)(lane + 32) : (int16_t)-1;
+}
+
+// One panel's search by one warp: Gauss-Jordan on up to 32 * NS slices of the
+// list, bit-reversed so that the leftmost column is the top bit. As in
+// eliminate_warp a warp maximum finds whether the column has a pivot and its
+// slice at once, and no step branches. Each slice keeps the set (record) of
+// pivots it absorbed, a pivot being named by its column: the pivot of column b
+// publishes its record with bit b added. Of the slices equal to the maximum, the
+// one with the largest record is the pivot (a second maximum, in flight together
+// with the next column's first); of several equal in both any may be, and the
+// one whose row ends up in prow is. The pivot's slice and set move to the pivot
+// slot of lane b, where later pivots clear their columns; the set ends as H_b.
+// A column is about 45 cycles; with a find-first and shuffles instead of the
+// maxima, and a branch where there is no pivot, it was 200.
+//
+// The loop runs eight columns per turn with the slices shifted up by eight after
+// each (what they shift out is zero in every candidate), so that its code stays
+// in the instruction cache: unrolled over 32 columns it ran half as fast.
+template <int NS, typename Smem>
+__device__ __forceinline__ uint32_t panel_search(Smem& sm, int16_t* prow, int nl, int p, int lane)
+{
+    uint32_t s[NS], c[NS];
+    uint32_t q = 0u;
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
+        s[j] = 32 * j + lane < nl ? __brev(sm.list[32 * j + lane]) : 0u;
+        c[j] = 0u;
+        q = max(q, s[j]);
+    }
+    q = __reduce_max_sync(0xffffffffu, q);
+    uint32_t ps = 0u, pc = 0u;  // lane b: the slice and set of column b's pivot
+    prow[lane] = -1;
+#pragma unroll 1
+    for (int b0 = 0; b0 < 32 && q; b0 += 8) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t L = 0x80000000u >> u;
+            const bool piv = q & L;
+            const uint32_t qs = q;
+            uint32_t rc = 0u, mx = 0u;
+            bool has[NS];
+#pragma unroll
+            for (int j = 0; j < NS; ++j) {
+                has[j] = s[j] & L;
+                rc = max(rc, s[j] == qs ? c[j] : 0u);
+                s[j] ^= has[j] ? qs : 0u;
+                mx = max(mx, s[j]);
+            }
+            const uint32_t own = __reduce_max_sync(0xffffffffu, rc);
+            q = __reduce_max_sync(0xffffffffu, mx);
+            const uint32_t qc = own ^ (1u << (b0 + u));
+#pragma unroll
+            for (int j = 0; j < NS; ++j) c[j] ^= has[j] ? qc : 0u;
+            const bool clears = piv && (ps & L);
+            ps ^= clears ? qs : 0u;
+            pc ^= clears ? qc : 0u;
+            if (piv && lane == b0 + u) {
+                ps = qs;
+                pc = qc;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < NS; ++j) s[j] <<= 8;
+        ps <<= 8;
+        q <<= 8;
+    }
+    const uint32_t cols = __ballot_sync(0xffffffffu, pc != 0u);
+    sm.Hcol[lane] = pc;
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
+        // a pivot absorbed itself, which leaves its own column alone in its record;
+        // so does a row whose start slice equals a pivot's, which is as good
+        const int col = __popc(c[j]) == 1 ? 31 - __clz(c[j]) : -1;
+        sm.kres[32 * j + lane] = (int16_t)col;
+        if (col >= 0) prow[col] = sm.listrow[32 * j + lane];
+    }
+    __syncwarp();
+    if (pc && HLF_IN_BOUNDS(32 * p + lane, (int)(sizeof sm.rowof / sizeof sm.rowof[0]), kSiteFactorSmem))
+        sm.rowof[32 * p + lane] = prow[lane];
+    if (lane == 0) {
+        sm.pivmask[p] |= cols;
+        sm.cols = cols;
+    }
+    return cols;
+}
+
+// W > 1: the elimination by panels of 32 columns, in a CTA of row threads (R rows
+// each: t, t + row threads, ...) and one more warp that searches.
+//
+// Per panel: (a) the row threads list the slices of the live rows; (b) the searching
+// warp finds the panel's pivots (panel_search); (c) T2 gets the combinations of the
+// pivots' start rows over 4 columns each; (d) every row is rebuilt as itself XOR
+// the start rows in its coefficient set, eight lookups a word. The reduced pivot
+// row of column b is the set H_b, and a row that is not one of the panel's
+// pivots, searched or not, absorbs the XOR of H over the pivot columns its start
+// slice has (nibble tables T1). The result has zeros on the panel's pivot columns
+// outside each pivot's own row and the same row space. Rows left over when the
+// search took only a part of the list can still hold bits in columns that got no
+// pivot; the panel is then searched again for them. Pivot columns are those of
+// the unique echelon form whatever the order, so nothing depends on the list's.
+//
+// The search of a panel needs one word of every row only, so (c) and (d) do that
+// word first and leave the others until the search of the next panel has begun:
+// the row threads finish them while the other warp searches.
+// `copy` ([W][stride], or null) receives A as it came; `meanwhile(warp, warps)` is
+// called by the row warps while the first panel is searched.
+template <int W, int R, int MAXN, typename F>
+__device__ void eliminate_panels(const uint64_t* __restrict__ A, int n, unsigned char* smem, uint64_t* copy,
+                                 F&& meanwhile)
+{
+    using Smem = FactorSmem<W, MAXN>;
+    Smem& sm = *reinterpret_cast<Smem*>(smem);
+    const int S = row_stride<W>(n);
+    uint64_t* rows = factor_rows<W, MAXN>(smem);  // [W][S]
+    uint64_t* T2 = rows + (size_t)W * S;          // [8][W][16]
+    const int lane = threadIdx.x & 31;
+    const int warp = warp_uniform(threadIdx.x >> 5);
+    const int rt = 32 * row_warps(blockDim.x >> 5);
+    const int npanels = (n + 31) >> 5;
+
+    for (int i = threadIdx.x; i < MAXN / 32; i += blockDim.x) sm.pivmask[i] = 0u;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) sm.rowof[i] = -1;
+    if (threadIdx.x < 2) sm.nlist[threadIdx.x] = 0;
+    if (threadIdx.x == 2) sm.nactive = 0;
     __syncthreads();
 
-    // ---- input checks: padding bits, then symmetry. A warp takes the 64 x 64
-    // blocks (I, J) and (J, I), I <= J, of the W x W block grid, transposes the
-    // first in registers and compares it with the second on the rows and
-    // columns below n.
-    int bad = 0;
+    if (warp == search_warp(blockDim.x >> 5)) {
+        for (int p = 0, round = 0; p < npanels; ++round) {
+            bar_elim(rt);  // the list is there
+            const int nl = warp_uniform(sm.nlist[round & 1]);
+            if (lane == 0) sm.nlist[(round + 1) & 1] = 0;
+            const int ncols = n - 32 * p < 32 ? n - 32 * p : 32;
+            uint32_t cols = 0u;
+            if (nl) {
+                const int cap = panel_cap(nl);
+                cols = cap == 32   ? panel_search<1>(sm, sm.prow[round & 1], nl, p, lane)
+                       : cap == 64 ? panel_search<2>(sm, sm.prow[round & 1], nl, p, lane)
+                                   : panel_search<4>(sm, sm.prow[round & 1], nl, p, lane);
+            }
+            if (panel_done(nl, cols, ncols)) ++p;
+            bar_elim(rt);             // the pivots are known
+            if (cols) bar_elim(rt);  // T1 and T2's first word are built
+        }
+        bar_elim(rt);
+        return;
+    }
+    if ((warp & 3) == 3) return;               // idle
+    const int tid = 32 * (warp - (warp >> 2)) + lane;  // the row thread's number
+
+    auto bar_rows = [&]() {
+        __syncwarp();
+        asm volatile("bar.sync 2, %0;" ::"r"(rt) : "memory");
+    };
+#pragma unroll 8
+    for (int i = tid; i < n * W; i += rt) {  // consecutive threads, consecutive words
+        const uint64_t x = A[i];
+        const int row = i / W, v = i % W;
+        rows[v * S + row] = x;
+        if (copy) copy[v * S + row] = x;
+    }
+    bool used[R];      // the row is a pivot row
+    uint32_t coef[R];  // the pivots it absorbs in the current panel
 #pragma unroll
     for (int j = 0; j < R; ++j) {
-        const int tail = n & 63;
-        if (tid + j * bs < n && tail && (row[j][W - 1] >> tail)) bad = HLF_ERR_PADDING;
+        used[j] = false;
+        coef[j] = 0u;
     }
+    bar_rows();
+    const int16_t* prow = sm.prow[0];  // the last panel's
+    // T2[(t, v, x)]: XOR of word v of the pivot rows of columns 4t + i, i over the bits of x
+    auto build = [&](int t, int v, int x) {
+        const uint64_t pr = *reinterpret_cast<const uint64_t*>(prow + 4 * t);
+        uint64_t acc = 0ull;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int row = (int16_t)(pr >> (16 * i));
+            if (((x >> i) & 1) && row >= 0 && HLF_IN_BOUNDS(row, n, kSiteFactorSmem)) acc ^= rows[v * S + row];
+        }
+        if (HLF_IN_BOUNDS((t * W + v) * 16 + x, 128 * W, kSiteFactorSmem)) T2[(t * W + v) * 16 + x] = acc;
+    };
+    auto update = [&](int row, uint32_t cf, int v) {
+        uint64_t* x = rows + v * S + row;
+        uint64_t a[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) a[t] = T2[(t * W + v) * 16 + ((cf >> (4 * t)) & 15u)];
+        *x ^= ((a[0] ^ a[1]) ^ (a[2] ^ a[3])) ^ ((a[4] ^ a[5]) ^ (a[6] ^ a[7]));
+    };
+    // Words w_from.. but w_done still lack the last panel's update. The rows that
+    // need it (on a grid, those near the panel) are listed and their words dealt to
+    // all row warps: 32 rows and kTaskWords words a task.
+    constexpr int kTaskWords = 4;
+    int w_from = W, w_done = 0;
+    auto finish = [&]() {
+        if (w_from + (w_done == w_from) >= W) return;  // uniform
+        for (int q = tid >> 4; q < 8 * (W - w_from); q += rt >> 4) {
+            const int v = w_from + (q >> 3);
+            if (v != w_done) build(q & 7, v, tid & 15);
+        }
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const unsigned m = __ballot_sync(0xffffffffu, coef[j] != 0u);
+            if (!m) continue;
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&sm.nactive, __popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
+            if (coef[j] && HLF_IN_BOUNDS(base, MAXN, kSiteFactorSmem))
+                sm.active[base] = make_uint2((uint32_t)(tid + j * rt), coef[j]);
+        }
+        bar_rows();
+        const int na = sm.nactive;
+        const int chunks = (na + 31) >> 5;
+        int ch = tid >> 5, v0 = w_from;
+        for (;;) {
+            while (ch >= chunks && v0 < W) {
+                ch -= chunks;
+                v0 += kTaskWords;
+            }
+            if (v0 >= W || !chunks) break;
+            const int e = 32 * ch + lane;
+            if (e < na) {
+                const uint2 rc = sm.active[e];
+                const uint64_t* tb[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) tb[t] = T2 + (t * W + v0) * 16 + ((rc.y >> (4 * t)) & 15u);
+                uint64_t* x = rows + v0 * S + rc.x;
+#pragma unroll 2
+                for (int i = 0; i < kTaskWords; ++i) {
+                    if (v0 + i >= W) break;
+                    if (v0 + i == w_done) continue;
+                    x[i * S] ^= ((tb[0][16 * i] ^ tb[1][16 * i]) ^ (tb[2][16 * i] ^ tb[3][16 * i])) ^
+                                ((tb[4][16 * i] ^ tb[5][16 * i]) ^ (tb[6][16 * i] ^ tb[7][16 * i]));
+                }
+            }
+            ch += rt >> 5;
+        }
+        w_from = W;
+    };
+    for (int p = 0, round = 0; p < npanels; ++round) {
+        const int w = p >> 1;
+        const int ncols = n - 32 * p < 32 ? n - 32 * p : 32;
+        const uint32_t in_n = ncols == 32 ? ~0u : (1u << ncols) - 1u;  // bits past n may be set in faulty input
+        uint32_t s[R];
+        int pos[R];
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const int row = tid + j * rt;
+            s[j] = row < n ? (uint32_t)(rows[w * S + row] >> (32 * (p & 1))) & in_n : 0u;
+            pos[j] = kPanelCap;
+            const bool live = s[j] != 0u && !used[j];
+            const unsigned m = __ballot_sync(0xffffffffu, live);
+            if (m) {
+                int base = 0;
+                if (lane == 0) base = atomicAdd(&sm.nlist[round & 1], __popc(m));
+                base = __shfl_sync(0xffffffffu, base, 0);
+                if (live) {
+                    pos[j] = base + __popc(m & ((1u << lane) - 1u));
+                    if (pos[j] < kPanelCap) {
+                        sm.list[pos[j]] = s[j];
+                        sm.listrow[pos[j]] = (int16_t)row;
+                    }
+                }
+            }
+        }
+        bar_elim(rt);  // the list is there
+        if (round == 0) meanwhile(tid >> 5, rt >> 5);
+        finish();
+        bar_elim(rt);  // the pivots are known
+        const int nl = sm.nlist[round & 1];
+        const uint32_t cols = nl ? sm.cols : 0u;
+        if (panel_done(nl, cols, ncols)) ++p;
+        if (!cols) continue;  // uniform: nothing absorbs anything
+        prow = sm.prow[round & 1];
+        if (tid == 0) sm.nactive = 0;
+        w_from = w;
+        w_done = (p >> 1) < W ? (p >> 1) : w;
+        for (int e = tid; e < 128; e += rt) build(e >> 4, w_done, e & 15);
+        for (int e = tid; e < 128; e += rt) {  // T1[(t, x)]: XOR of Hcol over the columns 4t + i, i over the bits of x
+            const uint4 h = *reinterpret_cast<const uint4*>(&sm.Hcol[4 * (e >> 4)]);
+            sm.T1[e] = ((e & 1 ? h.x : 0u) ^ (e & 2 ? h.y : 0u)) ^ ((e & 4 ? h.z : 0u) ^ (e & 8 ? h.w : 0u));
+        }
+        const int cap = panel_cap(nl);
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const int b = pos[j] < cap ? sm.kres[pos[j]] : -1;
+            // a pivot, unless its equal took the place
+            const bool now = b >= 0 && HLF_IN_BOUNDS(b, 32, kSiteFactorSmem) && prow[b] == tid + j * rt;
+            used[j] |= now;
+            coef[j] = now ? sm.Hcol[b] ^ (1u << b) : 0u;
+            if (now) s[j] = 0u;  // its set is known, not looked up
+        }
+        bar_elim(rt);  // T1 and T2's first word are built
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            if (s[j]) {
+#pragma unroll
+                for (int t = 0; t < 8; ++t) coef[j] ^= sm.T1[(t << 4) | ((s[j] >> (4 * t)) & 15u)];
+            }
+            if (coef[j]) update(tid + j * rt, coef[j], w_done);
+        }
+    }
+    finish();
+    bar_elim(rt);
+}
+
+// The input checks: padding bits, then symmetry, by warp `warp` of `nwarps`. A
+// warp takes the 64 x 64 blocks (I, J) and (J, I), I <= J, of the W x W block
+// grid, transposes the first in registers and compares it with the second on the
+// rows and columns below n. Returns this thread's verdict.
+template <int W>
+__device__ __forceinline__ int check_rows(const uint64_t* __restrict__ A, int n, int warp, int nwarps)
+{
+    const int lane = threadIdx.x & 31;
+    int bad = 0;
+    const int tail = n & 63;
+    if (tail)
+        for (int i = warp * 32 + lane; i < n; i += nwarps * 32)
+            if (A[(size_t)i * W + W - 1] >> tail) bad = HLF_ERR_PADDING;
     for (int pr = warp; pr < W * (W + 1) / 2; pr += nwarps) {
         int I = 0, rest = pr;  // pair index -> (I, J), I <= J < W
         while (rest >= W - I) {
@@ -153,7 +553,95 @@ __device__ int factor_block(const uint64_t* __restrict__ A, int n, const FactorO
         const uint64_t cm = cols >= 64 ? ~0ull : ((1ull << cols) - 1ull);
         if ((rb < n && ((p0 ^ q0) & cm)) || (rb + 32 < n && ((p1 ^ q1) & cm))) bad = max(bad, HLF_ERR_NOT_SYMMETRIC);
     }
-    if (bad) atomicMax(&sm.err, bad);
+    return bad;
+}
+
+// The rank, p_k and the rows of B_k from the pivot mask and rowof, by the whole CTA.
+template <int W, int MAXN>
+__device__ __forceinline__ int order_pivots(FactorSmem<W, MAXN>& sm, int n)
+{
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
+        const int cnt = 32 * lane < n ? __popc(sm.pivmask[lane]) : 0;
+        int incl = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += t;
+        }
+        if (32 * lane < n) sm.before[lane] = incl - cnt;
+        if (lane == 31) sm.rank = incl;
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < n; c += blockDim.x) {
+        const uint32_t m = sm.pivmask[c >> 5];
+        if (!((m >> (c & 31)) & 1u)) continue;
+        const int k = sm.before[c >> 5] + __popc(m & ((1u << (c & 31)) - 1u));
+        sm.pivcol[k] = (int16_t)c;
+        sm.rowk[k] = sm.rowof[c];
+    }
+    __syncthreads();
+    return sm.rank;
+}
+
+// Step (1)'s outputs: B_k in pivot order and the pivots (where asked for), the
+// enumeration table's rows below min(r, 64) and zeros from there to row `rows_to`.
+template <int W, int MAXN>
+__device__ __forceinline__ void write_basis(const FactorSmem<W, MAXN>& sm, const uint64_t* rows, int n, int r,
+                                            const FactorOut& o, int rows_to)
+{
+    const int S = row_stride<W>(n);
+    const int nb = r < HLF_MAX_VARYING ? r : HLF_MAX_VARYING;
+    const int last = o.basis ? r : nb;
+    for (int i = threadIdx.x; i < last * W; i += blockDim.x) {
+        const int k = i / W, v = i % W;
+        const int row = sm.rowk[k];
+        if (!HLF_IN_BOUNDS(row, S, kSiteFactorSmem)) continue;
+        const uint64_t x = rows[v * S + row];
+        if (o.basis) o.basis[i] = x;
+        if (k < nb) o.table[i] = x;
+    }
+    if (o.piv)
+        for (int k = threadIdx.x; k < r; k += blockDim.x) o.piv[k] = sm.pivcol[k];
+    for (int i = nb * W + threadIdx.x; i < rows_to * W; i += blockDim.x) o.table[i] = 0ull;
+}
+
+// Factor the n x n matrix A ([n][W] words, global) with the whole CTA. W > 1: R * 32
+// * row_warps(blockDim.x / 32) >= n; blockDim.x is a multiple of 32, at least 64.
+// n <= MAXN.
+// `smem` points to factor_smem_bytes<W, MAXN>(n, true) bytes of shared memory.
+// Writes o.table (always), o.basis, o.piv and o.ptable (when non-null) and
+// o.info[0] = status, o.info[1] = r (or -1 on a fault). Returns r, or -1.
+//
+// The steps around the elimination are chains of memory latencies, so they are
+// laid beside something else: the checks beside the elimination (a fault is seen
+// after it), the paper-order table (the last warp) and the outputs (the first)
+// beside the kernel vectors, and A is read from memory once.
+template <int W, int R, int MAXN>
+__device__ int factor_block(const uint64_t* __restrict__ A, int n, const FactorOut& o, unsigned char* smem)
+{
+    using Smem = FactorSmem<W, MAXN>;
+    Smem& sm = *reinterpret_cast<Smem*>(smem);
+    const int S = row_stride<W>(n);
+    uint64_t* rows = factor_rows<W, MAXN>(smem);
+    uint64_t* As = rows + (size_t)W * S + (W > 1 ? 8 * 16 * W : 0);  // A, [W][S]
+    const int tid = threadIdx.x;
+    const int lane = tid & 31;
+    const int warp = tid >> 5;
+    const int nwarps = blockDim.x >> 5;
+
+    if (tid == 0) sm.err = 0;
+    if (tid < W) sm.z0[tid] = 0;
+    __syncthreads();
+    auto check = [&](int w, int nw) {
+        if (const int bad = check_rows<W>(A, n, w, nw)) atomicMax(&sm.err, bad);
+    };
+    if constexpr (W == 1) {
+        if (warp_uniform(warp) == 0) eliminate_warp<MAXN>(A, n, smem, As);
+        else check(warp - 1, nwarps - 1);
+    } else {
+        eliminate_panels<W, R, MAXN>(A, n, smem, As, check);
+    }
     __syncthreads();
     if (sm.err) {
         const int e = sm.err;
@@ -164,159 +652,72 @@ __device__ int factor_block(const uint64_t* __restrict__ A, int n, const FactorO
         }
         return -1;
     }
-
-    // ---- (1) Gauss-Jordan elimination: B_k to s_rows[k][.], its pivot column to sm.pivcol[k]
-    int r;
-    {
-        bool used[R];
-        int my_k[R];
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-            used[j] = false;
-            my_k[j] = -1;
-        }
-        int rank = 0;
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-#pragma unroll 4  // 9-12% faster than rolled at n = 100..324
-            for (int b = 0; b < 64; ++b) {
-                const int c = (w << 6) + b;
-                if (c >= n) break;
-                const int buf = c & 1;
-                // this thread's lowest unused row with bit c, keyed (row << 5) | warp
-                int cand = kNone;
-#pragma unroll
-                for (int j = R - 1; j >= 0; --j)
-                    if (tid + j * bs < n && !used[j] && ((row[j][w] >> b) & 1ull)) cand = ((tid + j * bs) << 5) | warp;
-                const int wmin = __reduce_min_sync(0xffffffffu, cand);
-                if (wmin != kNone && cand == wmin) {  // this lane holds the warp's lowest candidate
-#pragma unroll
-                    for (int j = 0; j < R; ++j) {
-                        if (tid + j * bs != (wmin >> 5)) continue;
-#pragma unroll
-                        for (int v = w; v < W; ++v) sm.crow[buf][warp][v] = row[j][v];
-                    }
-                }
-                if (lane == 0) sm.first[buf][warp] = wmin;
-                __syncthreads();
-                int pk = lane < nwarps ? sm.first[buf][lane] : kNone;
-                pk = __reduce_min_sync(0xffffffffu, pk);
-                if (pk == kNone) continue;  // no pivot in column c (uniform)
-                const uint64_t* prow = sm.crow[buf][pk & 31];
-                const int p = pk >> 5;
-#pragma unroll
-                for (int j = 0; j < R; ++j) {
-                    if (tid + j * bs == p) {
-                        used[j] = true;
-                        my_k[j] = rank;
-                    }
-                }
-                if (tid == 0 && HLF_IN_BOUNDS(rank, HLF_MAX_N, kSiteFactorSmem)) sm.pivcol[rank] = c;
-                if constexpr (R == 1) {  // row p; its words below word w are zero
-                    uint64_t pv[W];
-#pragma unroll
-                    for (int v = w; v < W; ++v) pv[v] = prow[v];
-                    const uint64_t m = (tid != p && ((row[0][w] >> b) & 1ull)) ? ~0ull : 0ull;
-#pragma unroll
-                    for (int v = w; v < W; ++v) row[0][v] ^= pv[v] & m;
-                } else {
-#pragma unroll
-                    for (int j = 0; j < R; ++j) {
-                        if (tid + j * bs != p && ((row[j][w] >> b) & 1ull)) {
-#pragma unroll
-                            for (int v = w; v < W; ++v) row[j][v] ^= prow[v];
-                        }
-                    }
-                }
-                ++rank;
-            }
-        }
-        r = rank;
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-            if (!used[j] || !HLF_IN_BOUNDS(my_k[j], n, kSiteFactorSmem)) continue;
-#pragma unroll
-            for (int v = 0; v < W; ++v) s_rows[my_k[j] * SW + v] = row[j][v];
-        }
-    }
+    const int r = order_pivots(sm, n);
     const int nb = r < HLF_MAX_VARYING ? r : HLF_MAX_VARYING;
-    __syncthreads();
-
-    // ---- outputs of step (1): B_k in pivot order, pivots, enumeration table
-    for (int i = tid; i < r * W; i += bs) {
-        const uint64_t v = s_rows[(i / W) * SW + i % W];
-        if (o.basis) o.basis[i] = v;
-        if (i < nb * W) o.table[i] = v;
-    }
-    for (int i = nb * W + tid; i < kTableRows * W; i += bs) o.table[i] = 0ull;
-    for (int k = tid; k < r; k += bs) {
-        const int c = sm.pivcol[k];
-        if (o.piv) o.piv[k] = c;
-        atomicOr(&sm.pivmask[c >> 5], 1u << (c & 31));
-    }
-    __syncthreads();
-
-    // ---- (2)-(4): one warp per free column f
-    int err = 0;
-    for (int f = warp; f < n; f += nwarps) {
-        if ((sm.pivmask[f >> 5] >> (f & 31)) & 1u) continue;  // pivot column (uniform per warp)
-        const int fw = f >> 6;
-        const int fb = f & 63;
-        if (lane < W) sm.x[warp][lane] = lane == fw ? (1ull << fb) : 0ull;
-        __syncwarp();
-        // bit p_k of x_f is B_k[f]. pivcol ascends with k, so the lanes of a
-        // 32-row chunk that set bits of one word of x_f are contiguous, and
-        // an OR over them sets that word.
-        for (int k0 = 0; k0 < r; k0 += 32) {
-            const int k = k0 + lane;
-            const bool has = k < r && ((s_rows[k * SW + fw] >> fb) & 1ull);
-            const int pc = has ? sm.pivcol[k] : 0;
-            unsigned pending = __ballot_sync(0xffffffffu, has);
-            while (pending) {  // one word of x_f per pass (uniform)
-                const int wv = __shfl_sync(0xffffffffu, pc >> 6, __ffs(pending) - 1);
-                const bool mine = has && (pc >> 6) == wv;
-                const uint64_t bit = mine ? 1ull << (pc & 63) : 0ull;
-                const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)bit);
-                const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(bit >> 32));
-                if (lane == 0) sm.x[warp][wv] |= ((uint64_t)hi << 32) | lo;
-                pending &= ~__ballot_sync(0xffffffffu, mine);
-            }
-        }
-        __syncwarp();
-        unsigned acc = 0;
-        for (int i = lane; i < n; i += 32) {
-            if ((sm.x[warp][i >> 6] >> (i & 63)) & 1ull) {
-#pragma unroll
-                for (int v = 0; v < W; ++v) acc += __popcll(A[(size_t)i * W + v] & sm.x[warp][v]);
-            }
-        }
-        const unsigned q = __reduce_add_sync(0xffffffffu, acc) & 3u;
-        if (q & 1u) err = HLF_ERR_INTERNAL;  // q is even on Ker(A) for symmetric A
-        if (lane == 0 && (q >> 1))
-            atomicOr(reinterpret_cast<unsigned long long*>(&sm.z0[fw]), 1ull << fb);
-        __syncwarp();
-    }
-    if (err) atomicMax(&sm.err, err);
-    __syncthreads();
-    const int e = sm.err;
-    if (tid < W) o.table[kTableZ0Row * W + tid] = sm.z0[tid];
 
     // ---- the paper's own order (Section 2, Eq. 3; the counter of Section 4):
     // counter value t sets R_{p_j} = bit (r - j) of t, y = A R, z = y ^ z^a.
     // Bit l of t selects T_l = column p_{r-1-l} of A (0-based pivots), which is
     // row p_{r-1-l} since A is symmetric. With P_k = T_0 ^ ... ^ T_k, the Gray
     // walk over P visits z(t) in counter order, because bit l of t is the XOR
-    // of the Gray code's bits k >= l. One warp builds the prefix XORs.
-    if (o.ptable) {
-        if (warp == 0 && lane < W) {
-            uint64_t acc = 0;
-            for (int l = 0; l < nb; ++l) {
-                acc ^= A[(size_t)sm.pivcol[r - 1 - l] * W + lane];
-                o.ptable[l * W + lane] = acc;
+    // of the Gray code's bits k >= l. Lane l has rows l and l + 32, whose prefix
+    // XORs are two scans.
+    if (o.ptable && warp == nwarps - 1) {
+        for (int v = 0; v < W; ++v) {
+            uint64_t t0 = lane < nb ? As[v * S + sm.pivcol[r - 1 - lane]] : 0ull;
+            uint64_t t1 = lane + 32 < nb ? As[v * S + sm.pivcol[r - 33 - lane]] : 0ull;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint64_t u0 = __shfl_up_sync(0xffffffffu, t0, d);
+                const uint64_t u1 = __shfl_up_sync(0xffffffffu, t1, d);
+                if (lane >= d) {
+                    t0 ^= u0;
+                    t1 ^= u1;
+                }
+            }
+            t1 ^= __shfl_sync(0xffffffffu, t0, 31);
+            o.ptable[lane * W + v] = lane < nb ? t0 : 0ull;
+            o.ptable[(lane + 32) * W + v] = lane + 32 < nb ? t1 : 0ull;
+            if (lane == 0) o.ptable[64 * W + v] = 0ull;
+        }
+    }
+
+    // ---- (2)-(4): one warp per free column f, from the last warp but one down
+    int err = 0;
+    for (int f = nwarps - 1 - warp; f < n; f += nwarps) {
+        if ((sm.pivmask[f >> 5] >> (f & 31)) & 1u) continue;  // pivot column (uniform per warp)
+        const int fw = f >> 6;
+        const int fb = f & 63;
+        uint32_t x[2 * W];  // x_f, 32 bits a word
+#pragma unroll
+        for (int t = 0; t < 2 * W; ++t) {
+            const int c = 32 * t + lane;
+            const int row = c < n ? sm.rowof[c] : -1;
+            x[t] = __ballot_sync(0xffffffffu, row >= 0 && ((rows[fw * S + row] >> fb) & 1ull));
+            if (t == f >> 5) x[t] |= 1u << (f & 31);
+        }
+        unsigned acc = 0;
+#pragma unroll
+        for (int t = 0; t < 2 * W; ++t) {
+            if ((x[t] >> lane) & 1u) {
+#pragma unroll
+                for (int v = 0; v < W; ++v)
+                    acc += __popcll(As[v * S + 32 * t + lane] & (((uint64_t)x[2 * v + 1] << 32) | x[2 * v]));
             }
         }
-        for (int i = nb * W + tid; i < kTableRows * W; i += bs) o.ptable[i] = 0ull;
-        if (tid < W) o.ptable[kTableZ0Row * W + tid] = sm.z0[tid];
+        const unsigned q = __reduce_add_sync(0xffffffffu, acc) & 3u;
+        if (q & 1u) err = HLF_ERR_INTERNAL;  // q is even on Ker(A) for symmetric A
+        if (lane == 0 && (q >> 1))
+            atomicOr(reinterpret_cast<unsigned long long*>(&sm.z0[fw]), 1ull << fb);
+    }
+    if (err) atomicMax(&sm.err, err);
+
+    write_basis(sm, rows, n, r, o, kTableRows);
+    __syncthreads();
+    const int e = sm.err;
+    if (tid < W) {
+        o.table[kTableZ0Row * W + tid] = sm.z0[tid];
+        if (o.ptable) o.ptable[kTableZ0Row * W + tid] = sm.z0[tid];
     }
     if (tid == 0) {
         o.info[0] = e;
