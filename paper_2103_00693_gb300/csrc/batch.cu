@@ -88,6 +88,9 @@ constexpr size_t batch_smem_bytes()
     const size_t st = sizeof(Table<kBatchMaxW>) + sizeof(uint64_t) * (kTableRows - kStoreM) * kBatchMaxW +
                       sizeof(uint64_t) * NW * stage_words<kBatchMaxW>();
     m = st > m ? st : m;
+    // reduce chunks: table, seed tables
+    const size_t rd = sizeof(Table<kBatchMaxW>) + sizeof(SeedTable<kBatchMaxW>);
+    m = rd > m ? rd : m;
     return (m + 15) / 16 * 16;
 }
 static_assert(batch_smem_bytes<256>() <= 48 * 1024, "fits the default dynamic shared-memory limit");
@@ -121,7 +124,10 @@ __device__ void batch_reduce_chunk(const BatchArgs& a, int b, uint64_t first, ui
     constexpr int U = reduce_unroll(W);
     constexpr uint64_t kBlk = 1ull << U;
     Table<W>& t = *reinterpret_cast<Table<W>*>(smem);
-    load_table_hash_domain<W>(t, a.tables + (size_t)b * kTableSlot);
+    SeedTable<W>& st = *reinterpret_cast<SeedTable<W>*>(smem + sizeof(Table<W>));
+    const bool mixed = __syncthreads_or(load_table_hash_domain<W, U>(t, a.tables + (size_t)b * kTableSlot));
+    const int ntab = seed_tables_for(first + len - 1);
+    build_seed_table<W>(st, t, ntab);
     __syncthreads();
     // per-thread runs of whole 2^U blocks (chunks start at multiples of 2^U)
     const uint64_t per = ((len + T - 1) / T + kBlk - 1) & ~(kBlk - 1);
@@ -131,7 +137,9 @@ __device__ void batch_reduce_chunk(const BatchArgs& a, int b, uint64_t first, ui
     const uint64_t s = threadIdx.x * per;
     if (s < len) {
         cnt = min(per, len - s);
-        reduce_run<W, U>(t, first + s, cnt, acc);
+        uint64_t z[W];
+        seed_lookup<W>(st, ntab, first + s, z);
+        reduce_run_from<W, U>(t, mixed, first + s, cnt, z, acc);
     }
     block_reduce<W, T>(cnt, acc);
     if (threadIdx.x == 0 && cnt) {

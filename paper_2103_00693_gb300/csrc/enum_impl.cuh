@@ -36,12 +36,16 @@ __device__ __forceinline__ void load_table(Table<W>& t, const uint64_t* __restri
 }
 
 // The first layer of the SplitMix64 finalizer, L(x) = x ^ (x >> 30), is
-// linear over GF(2), so it commutes with the walk's XORs:
-// L(z(i+1)) = L(z(i)) ^ L(B_ctz(i+1)). The reduce therefore walks y = L(z) on
-// word 0, with a table whose word-0 entries are L(B_k) and L(z0), and hashes
-// y with the remaining layers (mix_tail). Hash values are bit-identical to
-// mix64(z); the XOR-fold of word 0 is taken in the L domain and mapped back
-// once with L^-1(y) = y ^ (y >> 30) ^ (y >> 60).
+// linear over GF(2), so it commutes with the walk's XORs and with the XOR that
+// chains the words: L(z(i+1)) = L(z(i)) ^ L(B_ctz(i+1)) and
+// L(h ^ w) = L(h) ^ L(w). The reduce therefore walks y = L(z) on every word, with a
+// table whose entries are L(B_k) and L(z0): word 0 skips the layer, and a later
+// word joins the layer of the chained hash as the third operand of its XORs.
+// Hash values are bit-identical to mix64 over z; the XOR-fold is taken in the L
+// domain and mapped back once with L^-1(y) = y ^ (y >> 30) ^ (y >> 60). Two of the
+// 16 ALU-pipe operations of a later word go away (cycles a warp of solutions
+// costs a scheduler: W = 2 64 -> 60, with the steps below; W = 7 253 -> 227,
+// W = 11 452 -> 358; 1024 grids of 1 to 4 words, batched: 2.10 -> 1.97 ms).
 __device__ __forceinline__ uint64_t mix_head(uint64_t x) { return x ^ (x >> 30); }
 __device__ __forceinline__ uint64_t mix_head_inv(uint64_t y) { return y ^ (y >> 30) ^ (y >> 60); }
 __device__ __forceinline__ uint64_t mix_tail(uint64_t y)
@@ -53,15 +57,20 @@ __device__ __forceinline__ uint64_t mix_tail(uint64_t y)
     return y;
 }
 
-// Table for the reduce: word 0 of every row (and of z0) taken through L.
-template <int W>
-__device__ __forceinline__ void load_table_hash_domain(Table<W>& t, const uint64_t* __restrict__ g)
+// Table for the reduce: every word of every row (and of z0) taken through L.
+// Returns whether this thread saw a row below U with a bit past word 0 (see
+// reduce_run_from); the callers OR it over the CTA while they synchronise.
+template <int W, int U>
+__device__ __forceinline__ bool load_table_hash_domain(Table<W>& t, const uint64_t* __restrict__ g)
 {
     uint64_t* d = &t.B[0][0];
+    bool mixed = false;
     for (int i = threadIdx.x; i < kTableTotalRows * W; i += blockDim.x) {
         const uint64_t v = __ldcg(g + i);
-        d[i] = (i % W == 0) ? mix_head(v) : v;
+        d[i] = mix_head(v);
+        mixed |= i < U * W && i % W != 0 && v != 0ull;
     }
+    return mixed;
 }
 
 // 64-bit shifts with PTX semantics: amounts of 64 give 0.
@@ -149,8 +158,8 @@ __device__ __forceinline__ void seed_lookup(const SeedTable<W>& st, int ntab, ui
     }
 }
 
-// Per-thread accumulator of the reduce, fed with solutions whose word 0 is in
-// the L domain (see load_table_hash_domain): sum of hashes and XOR-fold.
+// Per-thread accumulator of the reduce, fed with solutions in the L domain (see
+// load_table_hash_domain): sum of hashes and XOR-fold.
 template <int W>
 struct Acc {
     uint64_t hs;
@@ -161,26 +170,23 @@ struct Acc {
 #pragma unroll
         for (int w = 0; w < W; ++w) fold[w] = 0;
     }
-    __device__ __forceinline__ void consume(const uint64_t (&z)[W])
+    // The hash alone: for the solutions of whole aligned Gray blocks, whose
+    // XOR is zero (see reduce_run_from).
+    __device__ __forceinline__ void consume_hash(const uint64_t (&z)[W])
     {
         uint64_t h = mix_tail(z[0]);  // = mix64 of the solution's word 0
 #pragma unroll
-        for (int w = 1; w < W; ++w) h = mix64(h ^ z[w]);
+        for (int w = 1; w < W; ++w) h = mix_tail(mix_head(h) ^ z[w]);
         hs += h;
+    }
+    __device__ __forceinline__ void consume(const uint64_t (&z)[W])
+    {
+        consume_hash(z);
 #pragma unroll
         for (int w = 0; w < W; ++w) fold[w] ^= z[w];
     }
-    // The hash alone: for the solutions of whole aligned Gray blocks, whose
-    // XOR is zero (see reduce_run).
-    __device__ __forceinline__ void consume_hash(const uint64_t (&z)[W])
-    {
-        uint64_t h = mix_tail(z[0]);
-#pragma unroll
-        for (int w = 1; w < W; ++w) h = mix64(h ^ z[w]);
-        hs += h;
-    }
     // XOR-fold back in the solution domain (after all XOR reductions).
-    __device__ __forceinline__ uint64_t fold_word(int w) const { return w == 0 ? mix_head_inv(fold[0]) : fold[w]; }
+    __device__ __forceinline__ uint64_t fold_word(int w) const { return mix_head_inv(fold[w]); }
 };
 
 // The accumulator seen by whole aligned Gray blocks: hash only.
@@ -192,34 +198,40 @@ struct HashOnly {
 
 // 2^L consecutive solutions starting at an index that is a multiple of 2^L:
 // the reflected Gray code is (first half, flip bit L-1, second half), so the
-// step between the halves is row L-1, at a compile-time index. `Rows` is a
-// register array (W = 1) or the shared-memory table (W > 1, where register
-// copies of U rows of W words would cost more occupancy than they save).
-// `Sink` consumes each solution (the reduce accumulator, a histogram).
-template <int W, int L, typename Rows, typename Sink>
+// step between the halves is row L-1, at a compile-time index. `Rows` holds the
+// first NW words of each row: a register array where that is one word, else the
+// shared-memory table (register copies of U rows of W words would cost more
+// occupancy than they save). `Sink` consumes each solution.
+template <int W, int L, int NW, typename Rows, typename Sink>
 struct GrayBlock {
     static __device__ __forceinline__ void run(uint64_t (&z)[W], const Rows& Br, Sink& sink)
     {
-        GrayBlock<W, L - 1, Rows, Sink>::run(z, Br, sink);
-        xor_row<W>(z, Br[L - 1]);
-        GrayBlock<W, L - 1, Rows, Sink>::run(z, Br, sink);
+        GrayBlock<W, L - 1, NW, Rows, Sink>::run(z, Br, sink);
+#pragma unroll
+        for (int w = 0; w < NW; ++w) z[w] ^= Br[L - 1][w];
+        GrayBlock<W, L - 1, NW, Rows, Sink>::run(z, Br, sink);
     }
 };
-template <int W, typename Rows, typename Sink>
-struct GrayBlock<W, 0, Rows, Sink> {
+template <int W, int NW, typename Rows, typename Sink>
+struct GrayBlock<W, 0, NW, Rows, Sink> {
     static __device__ __forceinline__ void run(uint64_t (&z)[W], const Rows&, Sink& sink) { sink.consume(z); }
 };
 
-// The reduce of [i, i + len), len >= 1, with z = z(i) (word 0 in the L domain).
-// The solutions of an aligned block of 2^U
-// consecutive indices (U >= 2) are z_s ^ XOR_{k in S} B_k over all subsets S
-// of {0..U-1}: z_s and every B_k occur an even number of times, so their
-// XOR is zero (in the L domain too, L being linear). Whole blocks therefore
-// feed only the hash; the head and the tail of the run (partial blocks) feed
-// hash and fold. The fold is exact, and one 64-bit XOR per solution lighter.
+// The reduce of [i, i + len), len >= 1, with z = z(i) in the L domain.
+// The solutions of an aligned block of 2^U consecutive indices (U >= 2) are
+// z_s ^ XOR_{k in S} B_k over all subsets S of {0..U-1}: z_s and every B_k occur
+// an even number of times, so their XOR is zero (in the L domain too, L being
+// linear). Whole blocks therefore feed only the hash; the head and the tail of
+// the run (partial blocks) feed hash and fold. The fold is exact, and one 64-bit
+// XOR per solution lighter.
+//
+// `mixed`: some row below U has bits past word 0. Reduced rows are zero outside
+// their pivot and the free columns, so on grids, whose dependencies are local,
+// the first rows usually have none; the steps inside a block then touch word 0
+// only, held in registers.
 template <int W, int U>
-__device__ __forceinline__ void reduce_run_from(const Table<W>& t, uint64_t i, uint64_t len, uint64_t (&z)[W],
-                                                Acc<W>& acc)
+__device__ __forceinline__ void reduce_run_from(const Table<W>& t, bool mixed, uint64_t i, uint64_t len,
+                                                uint64_t (&z)[W], Acc<W>& acc)
 {
     static_assert(U >= 2, "a block of 2^U solutions XORs to zero only for U >= 2");
     constexpr uint64_t kBlk = 1ull << U;
@@ -231,19 +243,19 @@ __device__ __forceinline__ void reduce_run_from(const Table<W>& t, uint64_t i, u
     }
     if (len >= kBlk) {
         HashOnly<W> ho{acc};
-        if constexpr (W == 1) {
-            uint64_t Br[U][W];
+        if (W == 1 || !mixed) {
+            uint64_t Br[U][1];
 #pragma unroll
             for (int k = 0; k < U; ++k) Br[k][0] = t.B[k][0];
             do {
-                GrayBlock<W, U, uint64_t[U][W], HashOnly<W>>::run(z, Br, ho);
+                GrayBlock<W, U, 1, uint64_t[U][1], HashOnly<W>>::run(z, Br, ho);
                 len -= kBlk;
                 i += kBlk;
                 if (len) xor_row<W>(z, t.B[ctz64(i)]);  // ctz(i) >= U here
             } while (len >= kBlk);
         } else {
             do {
-                GrayBlock<W, U, uint64_t[kTableRows][W], HashOnly<W>>::run(z, t.B, ho);
+                GrayBlock<W, U, W, uint64_t[kTableRows][W], HashOnly<W>>::run(z, t.B, ho);
                 len -= kBlk;
                 i += kBlk;
                 if (len) xor_row<W>(z, t.B[ctz64(i)]);
@@ -256,15 +268,6 @@ __device__ __forceinline__ void reduce_run_from(const Table<W>& t, uint64_t i, u
         ++i;
         if (len) xor_row<W>(z, t.B[ctz64(i)]);
     }
-}
-
-template <int W, int U>
-__device__ __forceinline__ void reduce_run(const Table<W>& t, uint64_t i, uint64_t len, Acc<W>& acc)
-{
-    if (len == 0) return;
-    uint64_t z[W];
-    seed<W>(t, i, z);
-    reduce_run_from<W, U>(t, i, len, z, acc);
 }
 
 // Block-wide (count, hsum, fold) reduction over a CTA of THREADS threads;

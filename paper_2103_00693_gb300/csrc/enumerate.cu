@@ -53,8 +53,7 @@ __global__ void __launch_bounds__(T, min_ctas_for(W))
 {
     __shared__ Table<W> t;
     __shared__ SeedTable<W> st;
-    load_table_hash_domain<W>(t, table);
-    __syncthreads();
+    const bool mixed = __syncthreads_or(load_table_hash_domain<W, U>(t, table));
     build_seed_table<W>(st, t, ntab);
     __syncthreads();
     for (uint64_t item = blockIdx.x; item < n_chunks * parts; item += gridDim.x) {
@@ -72,7 +71,7 @@ __global__ void __launch_bounds__(T, min_ctas_for(W))
             uint64_t z[W];
             const uint64_t i = first + (lo - skip);
             seed_lookup<W>(st, ntab, i, z);
-            reduce_run_from<W, U>(t, i, cnt, z, acc);
+            reduce_run_from<W, U>(t, mixed, i, cnt, z, acc);
         }
         block_reduce<W, T>(cnt, acc);
         if (threadIdx.x != 0) continue;

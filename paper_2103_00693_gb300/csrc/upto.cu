@@ -47,14 +47,17 @@ __global__ void __launch_bounds__(kThreads) reduce_upto_kernel(const uint64_t* _
                                                                hlf_reduce* __restrict__ out)
 {
     __shared__ Table<W> t;
+    __shared__ SeedTable<W> st;
     __shared__ uint64_t s_count;
-    load_table_hash_domain<W>(t, table);
     if (threadIdx.x == 0) {
         const int32_t r = *reinterpret_cast<const volatile int32_t*>(info + 1);  // -1 after a fault
         s_count = r < 0 ? 0ull : (r >= 64 ? cap : (cap < (1ull << r) ? cap : (1ull << r)));
     }
-    __syncthreads();
+    const bool mixed = __syncthreads_or(load_table_hash_domain<W, U>(t, table));
     const uint64_t count = s_count;
+    const int ntab = seed_tables_for(cap - 1);
+    build_seed_table<W>(st, t, ntab);
+    __syncthreads();
     const uint64_t threads = (uint64_t)gridDim.x * blockDim.x;
     uint64_t per = (count + threads - 1) / threads;
     per = (per + (1ull << U) - 1) & ~((1ull << U) - 1);  // runs stay aligned to the Gray blocks
@@ -65,7 +68,9 @@ __global__ void __launch_bounds__(kThreads) reduce_upto_kernel(const uint64_t* _
     uint64_t cnt = 0;
     if (a < count) {
         cnt = min(per, count - a);
-        reduce_run<W, U>(t, a, cnt, acc);
+        uint64_t z[W];
+        seed_lookup<W>(st, ntab, a, z);
+        reduce_run_from<W, U>(t, mixed, a, cnt, z, acc);
     }
     block_reduce<W>(cnt, acc);
     if (threadIdx.x == 0 && cnt) {
