@@ -362,4 +362,110 @@ __device__ __forceinline__ void store_warp_coalesced(uint64_t* dst, const uint64
     __syncwarp();  // the stage is rewritten by the next call
 }
 
+// ------------------------------------------------------- storing by groups
+// A window is stored in groups of G consecutive solutions, one group a warp step:
+// G = 64 at W = 1 (a lane holds the pair z, z ^ B_0), 32 beyond. With m = log2 G,
+// g(G h + t) = (g(h) << m) ^ ((h & 1) << (m - 1)) ^ g(t), so stepping h -> h + 1
+// XORs the same row C_j = B_{m-1} ^ B_{m+j}, j = ctz(h + 1), into every lane.
+
+template <int W>
+struct Groups {
+    static constexpr int kPerLane = W == 1 ? 2 : 1;
+    static constexpr int kLog2 = W == 1 ? 6 : 5;
+    static constexpr uint64_t kSize = 32 * kPerLane;
+};
+
+// Groups [h_first, h_end) of the window [offset, offset + count), group h being the
+// indices G h + odd .. G h + odd + G - 1, and the indices before and after them.
+struct GroupPlan {
+    uint64_t n_head;      // [offset, offset + n_head)
+    uint64_t tail_first;  // [tail_first, tail_first + n_tail)
+    uint64_t n_tail;
+    uint64_t h_first, h_end;
+    uint32_t odd;
+};
+
+// odd (W = 1): pairs start at odd indices, so that they lie on 16 bytes where the
+// window's offset is odd; lane l then stores z(G h + 2 l + 1) and the next lane's
+// first solution (1.07 GB at an odd offset: 171 us, 198 with 8-byte stores). The window may end at 2^64 exactly, which wraps to 0.
+inline GroupPlan plan_groups(uint64_t offset, uint64_t count, uint64_t G, uint32_t odd)
+{
+    GroupPlan pl{};
+    pl.odd = odd;
+    const uint64_t end = offset + count;  // 0 for 2^64
+    const bool wraps = count != 0 && end == 0;
+    // first group at or after offset, and one past the last that ends by `end`
+    const uint64_t h_first = offset <= odd ? 0 : (offset - odd - 1) / G + 1;
+    const uint64_t h_end = wraps && !odd ? (0ull - G) / G + 1 : (end < odd && !wraps ? 0 : (end - odd) / G);
+    if (h_end <= h_first) {
+        pl.n_head = count;
+        return pl;
+    }
+    pl.h_first = h_first;
+    pl.h_end = h_end;
+    pl.n_head = h_first * G + odd - offset;
+    pl.tail_first = h_end * G + odd;  // wraps to 0 only when the tail is empty
+    pl.n_tail = count - pl.n_head - (h_end - h_first) * G;
+    return pl;
+}
+
+// z(G h + kPerLane * lane) for the 32 lanes of a warp. `row(k)` points to the W words
+// of B_k, z0 at row(kTableZ0Row). The part all lanes share is one XOR over the
+// warp, lane l bringing rows l and l + 32; the lane's own part has at most m rows.
+template <int W, typename Row>
+__device__ __forceinline__ void seed_group(Row row, uint64_t h, int lane, uint64_t (&z)[W])
+{
+    constexpr int M = Groups<W>::kLog2;
+    const uint64_t g = ((h ^ (h >> 1)) << M) ^ ((h & 1) << (M - 1));
+    const bool lo = (g >> lane) & 1u, hi = (g >> (lane + 32)) & 1u;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        const uint64_t a = (lo ? row(lane)[w] : 0ull) ^ (hi ? row(lane + 32)[w] : 0ull);
+        z[w] = ((uint64_t)__reduce_xor_sync(0xffffffffu, (uint32_t)(a >> 32)) << 32) |
+               __reduce_xor_sync(0xffffffffu, (uint32_t)a);
+        z[w] ^= row(kTableZ0Row)[w];
+    }
+    const int t = Groups<W>::kPerLane * lane;
+    const int gt = t ^ (t >> 1);
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+        const bool in = (gt >> k) & 1;
+#pragma unroll
+        for (int w = 0; w < W; ++w) z[w] ^= in ? row(k)[w] : 0ull;
+    }
+}
+
+// Groups [h, h1) of a window, h < h1, by one warp from the lanes' seeds: `dst` is the
+// output less offset * W words, `step(j)` points to C_j, `b0` is B_0's word (W = 1),
+// `stage` holds stage_words<W>() words of the warp (W > 1). W = 1 needs dst + odd on
+// 16 bytes or `pairs` false, W > 1 dst on 16 bytes.
+template <int W, typename Step, typename Check>
+__device__ __forceinline__ void store_groups(uint64_t (&z)[W], uint64_t h, uint64_t h1, uint32_t odd, uint64_t b0,
+                                             uint64_t* dst, uint64_t* stage, int lane, Step step, Check ok)
+{
+    constexpr uint64_t G = Groups<W>::kSize;
+    if constexpr (W == 1) {
+        for (;;) {
+            const uint64_t z1 = z[0] ^ b0;  // g(2t + 1) = g(2t) ^ 1
+            const uint64_t zn = z[0] ^ step(ctz64(h + 1))[0];
+            const uint64_t i = h * G + 2 * lane + odd;
+            if (odd) {  // warp-uniform
+                const uint64_t next = __shfl_sync(0xffffffffu, lane == 0 ? zn : z[0], (lane + 1) & 31);
+                if (ok(i, 2)) st_cs_v2(dst + i, z1, next);
+            } else {
+                if (ok(i, 2)) st_cs_v2(dst + i, z[0], z1);
+            }
+            if (++h == h1) break;
+            z[0] = zn;
+        }
+    } else {
+        for (;;) {
+            if (ok(h * G, G))  // warp-uniform
+                store_warp_coalesced<W, true>(dst + h * G * W, z, stage, lane);
+            if (++h == h1) break;
+            xor_row<W>(z, step(ctz64(h)));
+        }
+    }
+}
+
 }  // namespace hlf

@@ -20,16 +20,12 @@
 //                        Windows too short to give a full wave long runs are
 //                        bound by how many threads walk them: runs go down
 //                        to one Gray block.
-//   store_kernel         coalesced materialisation. Lane t of a warp owns
-//                        index G*h + S*t (+1), G = 32*S. With m = log2 G,
-//                          g(G h + t) = (g(h) << m) ^ ((h & 1) << (m-1)) ^ g(t),
-//                        so stepping h -> h+1 XORs the same row
-//                        C_j = B_{m-1} ^ B_{m+j}, j = ctz(h+1), into every
-//                        lane: one XOR per solution and a warp writes G
-//                        consecutive solutions per step (512 B at W = 1;
-//                        at W > 1 the lanes' solutions are restaged in
-//                        shared memory so that the warp writes its 32*W
-//                        words with consecutive lanes on consecutive words).
+//   store_kernel         coalesced materialisation by groups of 64 or 32
+//                        consecutive solutions a warp step (store_groups): one
+//                        XOR per solution, 512 B a step at W = 1; at W > 1 the
+//                        lanes' solutions are restaged in shared memory so that
+//                        the warp writes its 32*W words with consecutive lanes
+//                        on consecutive words. Bound by HBM stores.
 //   sample_kernel        z(i) at arbitrary indices, straight from the formula.
 
 #include "enum_impl.cuh"
@@ -95,21 +91,16 @@ __global__ void __launch_bounds__(T, min_ctas_for(W))
 
 struct StorePlan {
     uint64_t offset, count;
-    uint64_t n_head;       // ragged indices [offset, offset + n_head)
-    uint64_t tail_first;   // ragged indices [tail_first, offset + count)
-    uint64_t n_tail;
-    uint64_t h_first;      // groups [h_first, h_end) of G consecutive indices
-    uint64_t h_end;
-    uint64_t per_warp;     // groups per warp
+    GroupPlan g;
+    uint64_t per_warp;  // groups per warp
 };
 
-// S = solutions per lane (2 for W = 1, so a lane writes one 16-byte pair).
-template <int W, int S>
-__global__ void __launch_bounds__(kThreads) store_kernel(const uint64_t* __restrict__ table, StorePlan pl,
+template <int W>
+__global__ void __launch_bounds__(kThreads) store_kernel(const uint64_t* __restrict__ table,
+                                                         const __grid_constant__ StorePlan pl,
                                                          uint64_t* __restrict__ out)
 {
-    constexpr int G = 32 * S;
-    constexpr int M = (S == 2) ? 6 : 5;  // log2 G
+    constexpr int M = Groups<W>::kLog2;
     extern __shared__ __align__(16) uint64_t s_stage[];  // W > 1: [warps][stage_words<W>()]
     __shared__ Table<W> t;
     __shared__ uint64_t s_C[kTableRows - M][W];  // C_j = B_{M-1} ^ B_{M+j}
@@ -123,8 +114,8 @@ __global__ void __launch_bounds__(kThreads) store_kernel(const uint64_t* __restr
 
     const uint64_t gt = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     // ragged head and tail, one index per thread, from the definition
-    if (gt < pl.n_head + pl.n_tail) {
-        const uint64_t i = gt < pl.n_head ? pl.offset + gt : pl.tail_first + (gt - pl.n_head);
+    if (gt < pl.g.n_head + pl.g.n_tail) {
+        const uint64_t i = gt < pl.g.n_head ? pl.offset + gt : pl.g.tail_first + (gt - pl.g.n_head);
         uint64_t z[W];
         seed<W>(t, i, z);
         if (HLF_IN_BOUNDS(i - pl.offset, pl.count, kSiteStore)) {
@@ -132,37 +123,19 @@ __global__ void __launch_bounds__(kThreads) store_kernel(const uint64_t* __restr
             for (int w = 0; w < W; ++w) out[(i - pl.offset) * W + w] = z[w];
         }
     }
+    __syncwarp();
 
     const uint64_t wg = gt >> 5;
     const int lane = threadIdx.x & 31;
-    const uint64_t h0 = pl.h_first + wg * pl.per_warp;
-    if (wg * pl.per_warp >= pl.h_end - pl.h_first) return;
-    const uint64_t h1 = min(h0 + pl.per_warp, pl.h_end);
+    const uint64_t h0 = pl.g.h_first + wg * pl.per_warp;
+    if (wg * pl.per_warp >= pl.g.h_end - pl.g.h_first) return;
+    const uint64_t h1 = min(h0 + pl.per_warp, pl.g.h_end);
     uint64_t z[W];
-    seed<W>(t, h0 * G + (uint64_t)(S * lane), z);
-    // W = 1: a lane's pair starts at word out + (even index - offset); it is
-    // 16-byte aligned when the output's word index and the offset agree in parity
-    const bool even = (((reinterpret_cast<uintptr_t>(out) >> 3) ^ pl.offset) & 1) == 0;
-    for (uint64_t h = h0;;) {
-        if constexpr (S == 2) {
-            uint64_t* p = out + (h * G + (uint64_t)(S * lane) - pl.offset) * W;
-            const uint64_t z1 = z[0] ^ t.B[0][0];  // g(2t+1) = g(2t) ^ 1
-            if (HLF_RANGE_IN_BOUNDS(h * G + (uint64_t)(S * lane) - pl.offset, 2, pl.count, kSiteStore)) {
-                if (even) {
-                    st_cs_v2(p, z[0], z1);
-                } else {
-                    st_cs(p, z[0]);
-                    st_cs(p + 1, z1);
-                }
-            }
-        } else {  // W > 1: out is 16-byte aligned (checked by the callers); the check is warp-uniform
-            if (HLF_RANGE_IN_BOUNDS(h * G - pl.offset, G, pl.count, kSiteStore))
-                store_warp_coalesced<W, true>(out + (h * G - pl.offset) * W, z,
-                                              s_stage + (threadIdx.x >> 5) * stage_words<W>(), lane);
-        }
-        if (++h == h1) break;
-        xor_row<W>(z, s_C[ctz64(h)]);
-    }
+    seed_group<W>([&](int k) { return k == kTableZ0Row ? t.z0 : t.B[k]; }, h0, lane, z);
+    store_groups<W>(
+        z, h0, h1, pl.g.odd, t.B[0][0], out - pl.offset * W, s_stage + (threadIdx.x >> 5) * stage_words<W>(), lane,
+        [&](int j) { return s_C[j]; },
+        [&](uint64_t i, uint64_t len) { return HLF_RANGE_IN_BOUNDS(i - pl.offset, len, pl.count, kSiteStore); });
 }
 
 // ----------------------------------------------------------------- sample
@@ -302,60 +275,45 @@ hlf_status launch_reduce_w(const uint64_t* table, uint64_t offset, uint64_t chun
     return launch_reduce_u<W, reduce_unroll(W)>(table, offset, chunk, n_chunks, out, s);
 }
 
+// One wave of warps, each with consecutive groups; short windows give a warp one
+// group and spread the warps over the SMs (2^14 solutions of two words on one CTA
+// took 13 us, a group a warp on 64 CTAs takes 4).
 template <int W>
 hlf_status launch_store_w(const uint64_t* table, uint64_t offset, uint64_t count, uint64_t* out,
                           cudaStream_t s)
 {
-    constexpr int S = (W == 1) ? 2 : 1;
-    constexpr uint64_t G = 32 * S;
     StorePlan pl{};
     pl.offset = offset;
     pl.count = count;
-    // Full groups are [h_first * G, h_end * G). The window's end offset+count
-    // can be 2^64 exactly (r >= 64), which wraps to 0 in 64 bits; then the
-    // last group index is 2^(64 - log2 G).
-    const uint64_t end = offset + count;
-    const bool ends_at_2_64 = count != 0 && end == 0;
-    const uint64_t a0 = (offset + (G - 1)) & ~(G - 1);
-    const bool a0_wrapped = a0 < offset;
-    const uint64_t h_first = a0 / G;
-    const uint64_t h_end = ends_at_2_64 ? (0ull - G) / G + 1 : end / G;
-    const uint64_t groups = (!a0_wrapped && h_end > h_first) ? h_end - h_first : 0;
-    if (groups == 0) {
-        pl.n_head = count;
-        pl.n_tail = 0;
-        pl.tail_first = 0;
-        pl.h_first = pl.h_end = 0;
-    } else {
-        pl.n_head = a0 - offset;
-        pl.h_first = h_first;
-        pl.h_end = h_end;
-        pl.tail_first = h_end * G;  // wraps to 0 only when the tail is empty
-        pl.n_tail = count - pl.n_head - groups * G;
+    // W = 1: pairs on 16 bytes, whichever the parity of the window's first word
+    const uint32_t odd = W == 1 ? ((reinterpret_cast<uintptr_t>(out) >> 3) ^ offset) & 1 : 0;
+    pl.g = plan_groups(offset, count, Groups<W>::kSize, odd);
+    const uint64_t groups = pl.g.h_end - pl.g.h_first;
+    constexpr size_t smem_warp = W == 1 ? 0 : stage_words<W>() * sizeof(uint64_t);
+    constexpr size_t smem_max = smem_warp * (kThreads / 32);
+    static int fit[64] = {0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 64) return HLF_ERR_CUDA;
+    if (fit[dev] == 0) {
+        if (W > 1 && cudaFuncSetAttribute(store_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)smem_max) != cudaSuccess)
+            return HLF_ERR_CUDA;
+        fit[dev] = blocks_per_sm(store_kernel<W>, smem_max);
     }
-    const size_t smem = S == 1 ? (size_t)(kThreads / 32) * stage_words<W>() * sizeof(uint64_t) : 0;
-    if (S == 1) {
-        static bool attr_set[64] = {false};
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 64 && !attr_set[dev]) {
-            if (cudaFuncSetAttribute(store_kernel<W, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-                cudaSuccess)
-                return HLF_ERR_CUDA;
-            attr_set[dev] = true;
-        }
-    }
-    const uint64_t max_warps = (uint64_t)sm_count() * blocks_per_sm(store_kernel<W, S>, smem) * (kThreads / 32);
-    const uint64_t min_groups = 64;
-    uint64_t warps = (groups + min_groups - 1) / min_groups;
-    if (warps > max_warps) warps = max_warps;
+    const uint64_t sms = (uint64_t)sm_count();
+    const uint64_t max_warps = sms * fit[dev] * (kThreads / 32);
+    uint64_t warps = groups < max_warps ? groups : max_warps;
     if (warps == 0) warps = 1;
     pl.per_warp = groups ? (groups + warps - 1) / warps : 1;
-    const uint64_t ragged = pl.n_head + pl.n_tail;
+    if (groups) warps = (groups + pl.per_warp - 1) / pl.per_warp;
+    const uint64_t ragged = pl.g.n_head + pl.g.n_tail;
     uint64_t threads = warps * 32;
     if (threads < ragged) threads = ragged;
-    const unsigned blocks = (unsigned)((threads + kThreads - 1) / kThreads);
-    store_kernel<W, S><<<blocks, kThreads, smem, s>>>(table, pl, out);
+    uint64_t bd = (threads / sms + 31) / 32 * 32;
+    bd = bd < 64 ? 64 : (bd > kThreads ? kThreads : bd);
+    const unsigned blocks = (unsigned)((threads + bd - 1) / bd);
+    store_kernel<W><<<blocks, (unsigned)bd, smem_warp * (bd / 32), s>>>(table, pl, out);
     return cudaGetLastError() == cudaSuccess ? HLF_OK : HLF_ERR_CUDA;
 }
 

@@ -4,16 +4,13 @@
 // batching only schedules them together.
 //
 // The host cuts every window into warp tasks: task 0 of a window writes its
-// ragged head and tail (the indices before the first and after the last
-// multiple of G, seeded one by one from the definition), the other tasks
-// cover runs of up to kTaskGroups aligned groups of G consecutive indices
-// with the lane-interleaved Gray identity of enumerate.cu (one row XOR per
-// solution, a warp writes G consecutive solutions per step; solutions of
-// W > 1 words are restaged in shared memory so that the warp's stores are
-// coalesced). Warps take tasks
-// grid-stride and find their window by binary search over the task prefix
-// sums. The basis rows are read through the read-only cache: every lane of a
-// warp reads the same row, so each load is one broadcast.
+// ragged head and tail (the indices outside its groups, seeded one by one from
+// the definition), the other tasks cover runs of up to task_groups(W) groups
+// of consecutive indices (store_groups). Warps take tasks grid-stride and find
+// their window by binary search over the task prefix sums. A task's first step
+// rows are staged in shared memory, and its seed is one round of loads, every lane
+// bringing two rows. Seeded row by row from the table in global memory,
+// 48 windows (106 MB) in 64-group tasks took 68 us a call; now 52.
 
 #include <new>
 
@@ -22,17 +19,21 @@
 namespace hlf {
 namespace {
 
-constexpr uint64_t kTaskGroups = 64;
+// A task writes about 16 KB whatever W is, so that the last ones end together: with
+// 64 groups a task, one of W = 16 wrote 256 KB.
+__host__ __device__ constexpr uint64_t task_groups(uint32_t W) { return W == 1 ? 32 : 64 / W; }
+constexpr int kTaskRows = 6;  // step rows C_0 .. C_5 staged per warp: ctz(h) of 63 in 64 steps
 
 struct WinDesc {
     const uint64_t* table;  // [66][W]: B_0..B_64 (zero-padded), z0
     uint64_t* out;          // [count][W]
     uint64_t offset, count;
-    uint64_t n_head, tail_first, n_tail;  // ragged indices, as in StorePlan
-    uint64_t h_first, h_end;              // aligned groups [h_first, h_end)
-    uint64_t task_base;                   // tasks of earlier windows
+    GroupPlan g;
+    uint64_t task_base;  // tasks of earlier windows
     uint32_t W, ntasks;
 };
+
+constexpr int kWarpWords = stage_words<HLF_MAX_W>() + kTaskRows * HLF_MAX_W;  // shared words per warp
 
 template <int W>
 __device__ __forceinline__ void seed_g(const uint64_t* __restrict__ tab, uint64_t i, uint64_t (&z)[W])
@@ -51,12 +52,10 @@ __device__ __forceinline__ void seed_g(const uint64_t* __restrict__ tab, uint64_
 template <int W>
 __device__ void many_task(const WinDesc& d, uint64_t u, int lane, uint64_t* stage)
 {
-    constexpr int S = (W == 1) ? 2 : 1;
-    constexpr uint64_t G = 32 * S;
-    constexpr int M = (S == 2) ? 6 : 5;
-    if (u == 0 && d.n_head + d.n_tail) {
-        for (uint64_t e = lane; e < d.n_head + d.n_tail; e += 32) {
-            const uint64_t i = e < d.n_head ? d.offset + e : d.tail_first + (e - d.n_head);
+    constexpr int M = Groups<W>::kLog2;
+    if (u == 0 && d.g.n_head + d.g.n_tail) {
+        for (uint64_t e = lane; e < d.g.n_head + d.g.n_tail; e += 32) {
+            const uint64_t i = e < d.g.n_head ? d.offset + e : d.g.tail_first + (e - d.g.n_head);
             uint64_t z[W];
             seed_g<W>(d.table, i, z);
             if (HLF_IN_BOUNDS(i - d.offset, d.count, kSiteManyStore)) {
@@ -66,40 +65,34 @@ __device__ void many_task(const WinDesc& d, uint64_t u, int lane, uint64_t* stag
         }
         return;
     }
-    const uint64_t gt = (d.n_head + d.n_tail) ? u - 1 : u;
-    const uint64_t h0 = d.h_first + gt * kTaskGroups;
-    if (h0 >= d.h_end) return;
-    const uint64_t h1 = min(h0 + kTaskGroups, d.h_end);
+    const uint64_t gt = (d.g.n_head + d.g.n_tail) ? u - 1 : u;
+    const uint64_t h0 = d.g.h_first + gt * task_groups(W);
+    if (h0 >= d.g.h_end) return;
+    const uint64_t h1 = min(h0 + task_groups(W), d.g.h_end);
+    uint64_t* C = stage + stage_words<HLF_MAX_W>();  // [kTaskRows][W]
+    const uint64_t* tab = d.table;
+    for (int e = lane; e < kTaskRows * W; e += 32)
+        C[e] = __ldg(tab + (M - 1) * W + e % W) ^ __ldg(tab + M * W + e);
     uint64_t z[W];
-    seed_g<W>(d.table, h0 * G + (uint64_t)(S * lane), z);
-    const bool even = (d.offset & 1) == 0;  // outputs are 16-byte aligned (checked by the caller)
-    for (uint64_t h = h0;;) {
-        if constexpr (S == 2) {
-            uint64_t* p = d.out + (h * G + (uint64_t)(S * lane) - d.offset) * W;
-            const uint64_t z1 = z[0] ^ __ldg(d.table);  // g(2t+1) = g(2t) ^ 1
-            if (HLF_RANGE_IN_BOUNDS(h * G + (uint64_t)(S * lane) - d.offset, 2, d.count, kSiteManyStore)) {
-                if (even) {
-                    st_cs_v2(p, z[0], z1);
-                } else {
-                    st_cs(p, z[0]);
-                    st_cs(p + 1, z1);
-                }
-            }
-        } else {  // the check is warp-uniform
-            if (HLF_RANGE_IN_BOUNDS(h * G - d.offset, G, d.count, kSiteManyStore))
-                store_warp_coalesced<W, true>(d.out + (h * G - d.offset) * W, z, stage, lane);
-        }
-        if (++h == h1) break;
-        const int j = ctz64(h);
+    seed_group<W>([&](int k) { return tab + k * W; }, h0, lane, z);
+    __syncwarp();
+    uint64_t rare[W];  // a step row that is not staged
+    store_groups<W>(
+        z, h0, h1, d.g.odd, __ldg(tab), d.out - d.offset * W, stage, lane,
+        [&](int j) -> const uint64_t* {
+            if (j < kTaskRows) return C + j * W;
 #pragma unroll
-        for (int w = 0; w < W; ++w) z[w] ^= __ldg(d.table + (M - 1) * W + w) ^ __ldg(d.table + (M + j) * W + w);
-    }
+            for (int w = 0; w < W; ++w) rare[w] = __ldg(tab + (M - 1) * W + w) ^ __ldg(tab + (M + j) * W + w);
+            return rare;
+        },
+        [&](uint64_t i, uint64_t len) { return HLF_RANGE_IN_BOUNDS(i - d.offset, len, d.count, kSiteManyStore); });
+    __syncwarp();  // the staged rows are rewritten by the next task
 }
 
 __global__ void __launch_bounds__(kThreads, 2) many_kernel(const WinDesc* __restrict__ d, int k, uint64_t total_tasks)
 {
-    extern __shared__ __align__(16) uint64_t s_stage[];  // [warps][stage_words<16>()]
-    uint64_t* stage = s_stage + (threadIdx.x >> 5) * stage_words<HLF_MAX_W>();
+    extern __shared__ __align__(16) uint64_t s_stage[];  // [warps][kWarpWords]
+    uint64_t* stage = s_stage + (threadIdx.x >> 5) * kWarpWords;
     const int lane = threadIdx.x & 31;
     const uint64_t nwarps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     for (uint64_t t = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < total_tasks; t += nwarps) {
@@ -132,33 +125,15 @@ __global__ void __launch_bounds__(kThreads, 2) many_kernel(const WinDesc* __rest
     }
 }
 
-// Host-side cut of one window into tasks (the same plan as the single-window
-// store kernel).
+// Host-side cut of one window into tasks (outputs are 16-byte aligned, checked by
+// the caller).
 void plan_window(WinDesc& d, uint32_t W)
 {
-    const uint64_t G = W == 1 ? 64 : 32;
-    const int M = W == 1 ? 6 : 5;
-    const uint64_t end = d.offset + d.count;
-    const bool ends_at_2_64 = d.count != 0 && end == 0;
-    const uint64_t a0 = (d.offset + (G - 1)) & ~(G - 1);
-    const bool a0_wrapped = a0 < d.offset;
-    const uint64_t h_first = a0 / G;
-    const uint64_t h_end = ends_at_2_64 ? (1ull << (64 - M)) : end / G;
-    const uint64_t groups = (!a0_wrapped && h_end > h_first) ? h_end - h_first : 0;
-    if (groups == 0) {
-        d.n_head = d.count;
-        d.n_tail = 0;
-        d.tail_first = 0;
-        d.h_first = d.h_end = 0;
-    } else {
-        d.n_head = a0 - d.offset;
-        d.h_first = h_first;
-        d.h_end = h_end;
-        d.tail_first = h_end * G;
-        d.n_tail = d.count - d.n_head - groups * G;
-    }
+    const uint64_t G = W == 1 ? Groups<1>::kSize : Groups<2>::kSize;
+    d.g = plan_groups(d.offset, d.count, G, W == 1 ? d.offset & 1 : 0);
     d.W = W;
-    d.ntasks = (uint32_t)((d.n_head + d.n_tail ? 1 : 0) + (groups + kTaskGroups - 1) / kTaskGroups);
+    const uint64_t tg = task_groups(W);
+    d.ntasks = (uint32_t)((d.g.n_head + d.g.n_tail ? 1 : 0) + (d.g.h_end - d.g.h_first + tg - 1) / tg);
 }
 
 }  // namespace
@@ -255,7 +230,7 @@ hlf_status hlf_enumerate_store_many(hlf_many* m, hlf_handle* const* hs, const ui
     const uint64_t warps_cap = (uint64_t)hlf::sm_count() * 2 * (hlf::kThreads / 32);
     const uint64_t warps = tasks < warps_cap ? tasks : warps_cap;
     const unsigned blocks = (unsigned)((warps * 32 + hlf::kThreads - 1) / hlf::kThreads);
-    constexpr size_t smem = (size_t)(hlf::kThreads / 32) * hlf::stage_words<HLF_MAX_W>() * sizeof(uint64_t);
+    constexpr size_t smem = (size_t)(hlf::kThreads / 32) * hlf::kWarpWords * sizeof(uint64_t);
     hlf::many_kernel<<<blocks, hlf::kThreads, smem, s>>>(m->dev[b], used, tasks);
     if (cudaGetLastError() != cudaSuccess) return HLF_ERR_CUDA;
     if (cudaEventRecord(m->done[b], s) != cudaSuccess) return HLF_ERR_CUDA;
