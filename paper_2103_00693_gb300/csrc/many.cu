@@ -3,14 +3,17 @@
 // stage-2 materialisation of hlf_enumerate_store (Section 2, Fig. 1(c)); the
 // batching only schedules them together.
 //
-// The host cuts every window into warp tasks: task 0 of a window writes its
-// ragged head and tail (the indices outside its groups, seeded one by one from
-// the definition), the other tasks cover runs of up to task_groups(W) groups
-// of consecutive indices (store_groups). Warps take tasks grid-stride and find
-// their window by binary search over the task prefix sums. A task's first step
-// rows are staged in shared memory, and its seed is one round of loads, every lane
-// bringing two rows. Seeded row by row from the table in global memory,
-// 48 windows (106 MB) in 64-group tasks took 68 us a call; now 52.
+// The host cuts every window into tasks of about 4 KB of output: task 0 of a window
+// writes its ragged head and tail (the indices outside its groups, seeded one by
+// one from the definition), the others cover task_groups(W) groups of consecutive
+// indices each. A warp takes an equal run of tasks, finds its first window by binary
+// search over the task prefix sums, and stores the groups of each window in the run
+// in one walk (store_groups), so that it seeds itself once a window: a seed is one
+// round of loads, every lane bringing two rows, and the window's first step rows are
+// staged in shared memory.
+// 48 windows of 106 MB: the kernel took 69 us with 64-group tasks taken one by one
+// and seeded row by row from global memory, 52 with 16 KB tasks one by one, and takes
+// about 33 now; calls in a row are bound by the host's 50 us a call.
 
 #include <new>
 
@@ -19,9 +22,8 @@
 namespace hlf {
 namespace {
 
-// A task writes about 16 KB whatever W is, so that the last ones end together: with
-// 64 groups a task, one of W = 16 wrote 256 KB.
-__host__ __device__ constexpr uint64_t task_groups(uint32_t W) { return W == 1 ? 32 : 64 / W; }
+// A task is the unit that the warps' shares differ by.
+__host__ __device__ constexpr uint64_t task_groups(uint32_t W) { return W == 1 ? 8 : (16 + W - 1) / W; }
 constexpr int kTaskRows = 6;  // step rows C_0 .. C_5 staged per warp: ctz(h) of 63 in 64 steps
 
 struct WinDesc {
@@ -49,26 +51,30 @@ __device__ __forceinline__ void seed_g(const uint64_t* __restrict__ tab, uint64_
     }
 }
 
+// Tasks [u, u1) of window d by one warp.
 template <int W>
-__device__ void many_task(const WinDesc& d, uint64_t u, int lane, uint64_t* stage)
+__device__ void many_tasks(const WinDesc& d, uint64_t u, uint64_t u1, int lane, uint64_t* stage)
 {
     constexpr int M = Groups<W>::kLog2;
-    if (u == 0 && d.g.n_head + d.g.n_tail) {
-        for (uint64_t e = lane; e < d.g.n_head + d.g.n_tail; e += 32) {
-            const uint64_t i = e < d.g.n_head ? d.offset + e : d.g.tail_first + (e - d.g.n_head);
-            uint64_t z[W];
-            seed_g<W>(d.table, i, z);
-            if (HLF_IN_BOUNDS(i - d.offset, d.count, kSiteManyStore)) {
+    const uint64_t ragged = d.g.n_head + d.g.n_tail;
+    if (ragged) {
+        if (u == 0)
+            for (uint64_t e = lane; e < ragged; e += 32) {
+                const uint64_t i = e < d.g.n_head ? d.offset + e : d.g.tail_first + (e - d.g.n_head);
+                uint64_t z[W];
+                seed_g<W>(d.table, i, z);
+                if (HLF_IN_BOUNDS(i - d.offset, d.count, kSiteManyStore)) {
 #pragma unroll
-                for (int w = 0; w < W; ++w) d.out[(i - d.offset) * W + w] = z[w];
+                    for (int w = 0; w < W; ++w) d.out[(i - d.offset) * W + w] = z[w];
+                }
             }
-        }
-        return;
+        __syncwarp();
+        u -= u != 0;  // task t > 0 covers the groups of index t - 1
+        --u1;
     }
-    const uint64_t gt = (d.g.n_head + d.g.n_tail) ? u - 1 : u;
-    const uint64_t h0 = d.g.h_first + gt * task_groups(W);
-    if (h0 >= d.g.h_end) return;
-    const uint64_t h1 = min(h0 + task_groups(W), d.g.h_end);
+    const uint64_t h0 = d.g.h_first + u * task_groups(W);
+    const uint64_t h1 = min(d.g.h_first + u1 * task_groups(W), d.g.h_end);
+    if (h0 >= h1) return;
     uint64_t* C = stage + stage_words<HLF_MAX_W>();  // [kTaskRows][W]
     const uint64_t* tab = d.table;
     for (int e = lane; e < kTaskRows * W; e += 32)
@@ -86,41 +92,46 @@ __device__ void many_task(const WinDesc& d, uint64_t u, int lane, uint64_t* stag
             return rare;
         },
         [&](uint64_t i, uint64_t len) { return HLF_RANGE_IN_BOUNDS(i - d.offset, len, d.count, kSiteManyStore); });
-    __syncwarp();  // the staged rows are rewritten by the next task
+    __syncwarp();  // the staged rows are rewritten for the next window
 }
 
-__global__ void __launch_bounds__(kThreads, 2) many_kernel(const WinDesc* __restrict__ d, int k, uint64_t total_tasks)
+__global__ void __launch_bounds__(kThreads, 2) many_kernel(const WinDesc* __restrict__ d, int k, uint64_t total_tasks,
+                                                           uint64_t per_warp)
 {
     extern __shared__ __align__(16) uint64_t s_stage[];  // [warps][kWarpWords]
     uint64_t* stage = s_stage + (threadIdx.x >> 5) * kWarpWords;
     const int lane = threadIdx.x & 31;
-    const uint64_t nwarps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    for (uint64_t t = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < total_tasks; t += nwarps) {
-        int lo = 0, hi = k - 1;  // last window with task_base <= t
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (d[mid].task_base <= t) lo = mid;
-            else hi = mid - 1;
-        }
+    uint64_t t = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp;
+    const uint64_t t1 = min(t + per_warp, total_tasks);
+    if (t >= t1) return;
+    int lo = 0, hi = k - 1;  // last window with task_base <= t
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (d[mid].task_base <= t) lo = mid;
+        else hi = mid - 1;
+    }
+    for (; t < t1; ++lo) {
         const WinDesc& w = d[lo];
         const uint64_t u = t - w.task_base;
+        const uint64_t u1 = min(t1 - w.task_base, (uint64_t)w.ntasks);
+        t = w.task_base + u1;
         switch (w.W) {
-        case 1: many_task<1>(w, u, lane, stage); break;
-        case 2: many_task<2>(w, u, lane, stage); break;
-        case 3: many_task<3>(w, u, lane, stage); break;
-        case 4: many_task<4>(w, u, lane, stage); break;
-        case 5: many_task<5>(w, u, lane, stage); break;
-        case 6: many_task<6>(w, u, lane, stage); break;
-        case 7: many_task<7>(w, u, lane, stage); break;
-        case 8: many_task<8>(w, u, lane, stage); break;
-        case 9: many_task<9>(w, u, lane, stage); break;
-        case 10: many_task<10>(w, u, lane, stage); break;
-        case 11: many_task<11>(w, u, lane, stage); break;
-        case 12: many_task<12>(w, u, lane, stage); break;
-        case 13: many_task<13>(w, u, lane, stage); break;
-        case 14: many_task<14>(w, u, lane, stage); break;
-        case 15: many_task<15>(w, u, lane, stage); break;
-        default: many_task<16>(w, u, lane, stage); break;
+        case 1: many_tasks<1>(w, u, u1, lane, stage); break;
+        case 2: many_tasks<2>(w, u, u1, lane, stage); break;
+        case 3: many_tasks<3>(w, u, u1, lane, stage); break;
+        case 4: many_tasks<4>(w, u, u1, lane, stage); break;
+        case 5: many_tasks<5>(w, u, u1, lane, stage); break;
+        case 6: many_tasks<6>(w, u, u1, lane, stage); break;
+        case 7: many_tasks<7>(w, u, u1, lane, stage); break;
+        case 8: many_tasks<8>(w, u, u1, lane, stage); break;
+        case 9: many_tasks<9>(w, u, u1, lane, stage); break;
+        case 10: many_tasks<10>(w, u, u1, lane, stage); break;
+        case 11: many_tasks<11>(w, u, u1, lane, stage); break;
+        case 12: many_tasks<12>(w, u, u1, lane, stage); break;
+        case 13: many_tasks<13>(w, u, u1, lane, stage); break;
+        case 14: many_tasks<14>(w, u, u1, lane, stage); break;
+        case 15: many_tasks<15>(w, u, u1, lane, stage); break;
+        default: many_tasks<16>(w, u, u1, lane, stage); break;
         }
     }
 }
@@ -228,10 +239,11 @@ hlf_status hlf_enumerate_store_many(hlf_many* m, hlf_handle* const* hs, const ui
     // Two CTAs per SM keep HBM busy for stores and leave room on every SM for
     // the factorisations a serving loop runs alongside.
     const uint64_t warps_cap = (uint64_t)hlf::sm_count() * 2 * (hlf::kThreads / 32);
-    const uint64_t warps = tasks < warps_cap ? tasks : warps_cap;
+    const uint64_t per_warp = (tasks + warps_cap - 1) / warps_cap;
+    const uint64_t warps = (tasks + per_warp - 1) / per_warp;
     const unsigned blocks = (unsigned)((warps * 32 + hlf::kThreads - 1) / hlf::kThreads);
     constexpr size_t smem = (size_t)(hlf::kThreads / 32) * hlf::kWarpWords * sizeof(uint64_t);
-    hlf::many_kernel<<<blocks, hlf::kThreads, smem, s>>>(m->dev[b], used, tasks);
+    hlf::many_kernel<<<blocks, hlf::kThreads, smem, s>>>(m->dev[b], used, tasks, per_warp);
     if (cudaGetLastError() != cudaSuccess) return HLF_ERR_CUDA;
     if (cudaEventRecord(m->done[b], s) != cudaSuccess) return HLF_ERR_CUDA;
     // every handle read by this launch must outlive it (hlf_destroy waits)
