@@ -465,7 +465,9 @@ hlf_status launch_dense2_k(const uint64_t* table, int n, uint64_t offset, uint64
 // registers and stores them straight to global memory, so a warp writes 256
 // consecutive bytes per store instruction and nothing is staged; per block a
 // lane spends about four instructions per word it owns (load, 64-bit XOR,
-// store).
+// store). A CTA's first rows cost it a few microseconds, which counts in short
+// windows: formed word by word, two tiles each, 2^25 solutions of 100 bits (419 MB)
+// took 88 us; with each tile formed once, 81.
 constexpr int kD3J = 8;
 constexpr int kD3Threads = 256;
 constexpr int kD3Warps = kD3Threads / 32;
@@ -598,14 +600,30 @@ __global__ void __launch_bounds__(kD3Threads, W == 3 ? 4 : (W == 4 ? 3 : (MW > 4
         s_C[j][w] = mb + j < kTableRows ? t.B[mb - 1][w] ^ t.B[mb + j][w] : 0ull;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < 2 * kD3J * K; i += blockDim.x) {
-        const int row = i / K, q = i % K;
-        const int j = row < kD3J ? row : 0, jn = row < kD3J ? 0 : row - kD3J;
-        const uint64_t x = tile_word<W>(s_C[j], n, (uint32_t)q);
-        const uint64_t y = q + 1 < K ? tile_word<W>(s_C[j], n, (uint32_t)q + 1) : tile_word<W>(s_C[jn], n, 0);
-        s_S[i] = funnel(x, y, b);
+    // Thread q forms word q of the rows (K <= kD3Threads): first the tiles T_j, in
+    // the place of the odd blocks' rows, then the step rows from neighbouring words.
+    // The odd blocks' rows differ from row 0 in their last word only.
+    const uint32_t q0 = threadIdx.x;
+    if (q0 < (uint32_t)K) {
+        for (int j = 0; j < kD3J; ++j) s_S[(kD3J + j) * K + q0] = tile_word<W>(s_C[j], n, q0);
+        s_S0[q0] = group_base_word<W>(t, n, mb, q0);
     }
-    for (int q = threadIdx.x; q < K; q += blockDim.x) s_S0[q] = group_base_word<W>(t, n, mb, (uint32_t)q);
+    __syncthreads();
+    uint64_t odd[kD3J];
+    if (q0 < (uint32_t)K) {
+        const uint64_t* T = s_S + kD3J * K;
+        const bool last = q0 + 1 == (uint32_t)K;
+        const uint64_t x0 = T[q0];
+#pragma unroll
+        for (int j = 0; j < kD3J; ++j) {
+            s_S[j * K + q0] = funnel(T[j * K + q0], last ? T[0] : T[j * K + q0 + 1], b);
+            odd[j] = funnel(x0, last ? T[j * K] : T[q0 + 1], b);
+        }
+    }
+    __syncthreads();
+    if (q0 < (uint32_t)K)
+#pragma unroll
+        for (int j = 0; j < kD3J; ++j) s_S[(kD3J + j) * K + q0] = odd[j];
     __syncthreads();
 
     const int lane = threadIdx.x & 31;
@@ -614,18 +632,16 @@ __global__ void __launch_bounds__(kD3Threads, W == 3 ? 4 : (W == 4 ? 3 : (MW > 4
     if (k0 >= pl.groups) return;
     const uint64_t k1 = min(k0 + pl.per_warp, pl.groups);
     const uint64_t H0 = pl.Hw + k0;  // < 2^(64 - m)
-    {  // D(H0): every lane forms it; lane w < W publishes word w
-        uint64_t g = ((H0 ^ (H0 >> 1)) << mb) | ((H0 & 1ull) << (mb - 1));
-        uint64_t D[W];
+    {  // D(H0): one XOR over the warp, lane l bringing rows l and l + 32; lane w keeps word w
+        const uint64_t g = ((H0 ^ (H0 >> 1)) << mb) | ((H0 & 1ull) << (mb - 1));
+        const bool lo = (g >> lane) & 1u, hi = (g >> (lane + 32)) & 1u;
 #pragma unroll
-        for (int w = 0; w < W; ++w) D[w] = 0;
-        while (g) {
-            xor_row<W>(D, t.B[__ffsll((long long)g) - 1]);
-            g &= g - 1;
+        for (int w = 0; w < W; ++w) {
+            const uint64_t a = (lo ? t.B[lane][w] : 0ull) ^ (hi ? t.B[lane + 32][w] : 0ull);
+            const uint32_t dl = __reduce_xor_sync(0xffffffffu, (uint32_t)a);
+            const uint32_t dh = __reduce_xor_sync(0xffffffffu, (uint32_t)(a >> 32));
+            if (lane == w) s_D[warp * W + w] = ((uint64_t)dh << 32) | dl;
         }
-#pragma unroll
-        for (int w = 0; w < W; ++w)
-            if (lane == w) s_D[warp * W + w] = D[w];
         __syncwarp();
     }
     // G'(H0): f of consecutive words of G(H0), the last with G(H0 + 1)[0]
