@@ -124,8 +124,11 @@ struct SeedTable {
 // Tables covering the index bits that [0, last] uses.
 __host__ __device__ inline int seed_tables_for(uint64_t last)
 {
-    int bits = 1;
-    while (bits < 64 && (last >> bits)) ++bits;
+#ifdef __CUDA_ARCH__
+    const int bits = 64 - __clzll((long long)(last | 1));
+#else
+    const int bits = 64 - __builtin_clzll(last | 1);
+#endif
     return (bits + 3) / 4;
 }
 

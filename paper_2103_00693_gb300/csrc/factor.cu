@@ -75,6 +75,7 @@ constexpr int kWorkDone = 18;     // work[18] = CTAs of factor_kvec_kernel done
 constexpr int kWorkMask = 32;     // work[32..64) = the pivot columns, one bit each
 constexpr int kKvecCtas = 256;    // CTAs of factor_kvec_kernel (one free column at a time each)
 static_assert(kWorkMask + HLF_MAX_N / 32 <= kFactorWorkWords, "the pivot mask fits the scratch words");
+static_assert(kWorkDone < kFactorDevInfo && kFactorDevInfo + 2 <= kWorkMask, "the scratch words do not overlap");
 static_assert(kChkCtas <= kWorkR, "one status slot per checking CTA");
 
 // Step (1) for the whole CTA: the reduced row echelon form, pivots and the
@@ -255,8 +256,7 @@ __global__ void __launch_bounds__(256) factor_kvec_kernel(const uint64_t* __rest
         int st = 0;
         for (int k = 0; k < n_chk; ++k) st = max(st, __ldcg(o.work + k));
         if (!st) st = __ldcg(o.work + kWorkInternal);
-        o.info[0] = st;
-        o.info[1] = st ? -1 : r;
+        write_info(o, st, st ? -1 : r);
     }
 }
 

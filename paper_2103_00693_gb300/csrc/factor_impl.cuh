@@ -556,6 +556,16 @@ __device__ __forceinline__ int check_rows(const uint64_t* __restrict__ A, int n,
     return bad;
 }
 
+__device__ __forceinline__ void write_info(const FactorOut& o, int status, int r)
+{
+    o.info[0] = status;
+    o.info[1] = r;
+    if (o.work) {
+        o.work[kFactorDevInfo] = status;
+        o.work[kFactorDevInfo + 1] = r;
+    }
+}
+
 // The rank, p_k and the rows of B_k from the pivot mask and rowof, by the whole CTA.
 template <int W, int MAXN>
 __device__ __forceinline__ int order_pivots(FactorSmem<W, MAXN>& sm, int n)
@@ -646,10 +656,7 @@ __device__ int factor_block(const uint64_t* __restrict__ A, int n, const FactorO
     if (sm.err) {
         const int e = sm.err;
         __syncthreads();
-        if (tid == 0) {
-            o.info[0] = e;
-            o.info[1] = -1;
-        }
+        if (tid == 0) write_info(o, e, -1);
         return -1;
     }
     const int r = order_pivots(sm, n);
@@ -719,10 +726,7 @@ __device__ int factor_block(const uint64_t* __restrict__ A, int n, const FactorO
         o.table[kTableZ0Row * W + tid] = sm.z0[tid];
         if (o.ptable) o.ptable[kTableZ0Row * W + tid] = sm.z0[tid];
     }
-    if (tid == 0) {
-        o.info[0] = e;
-        o.info[1] = e ? -1 : r;
-    }
+    if (tid == 0) write_info(o, e, e ? -1 : r);
     __syncthreads();  // shared memory may be reused by the caller
     return e ? -1 : r;
 }

@@ -182,6 +182,12 @@ hlf_status ensure_rank(hlf_handle* h)
     return HLF_OK;
 }
 
+// status and rank as the factor kernel left them in device memory
+const int32_t* dev_info(const hlf_handle* h)
+{
+    return reinterpret_cast<const int32_t*>(h->dmem) + hlf::kFactorDevInfo;
+}
+
 const uint64_t* enum_table(const hlf_handle* h) { return h->order == HLF_ORDER_PAPER ? h->ptable : h->table; }
 
 // Is [offset, offset + count) inside [0, 2^min(r, 64))?
@@ -496,7 +502,7 @@ hlf_status hlf_enumerate_store_upto(hlf_handle* h, uint64_t cap, uint64_t* out_d
     if (cap == 0) return HLF_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (cudaStreamWaitEvent(s, h->factored, 0) != cudaSuccess) return HLF_ERR_CUDA;
-    return after_launch(h, hlf::launch_store_upto(enum_table(h), h->W, h->info_dev, cap, out_dev, s), s);
+    return after_launch(h, hlf::launch_store_upto(enum_table(h), h->W, dev_info(h), cap, out_dev, s), s);
 }
 
 hlf_status hlf_enumerate_reduce_upto(hlf_handle* h, uint64_t cap, hlf_reduce* red_dev, void* stream)
@@ -509,7 +515,7 @@ hlf_status hlf_enumerate_reduce_upto(hlf_handle* h, uint64_t cap, hlf_reduce* re
     if (cudaStreamWaitEvent(s, h->factored, 0) != cudaSuccess) return HLF_ERR_CUDA;
     if (cudaMemsetAsync(red_dev, 0, sizeof(hlf_reduce), s) != cudaSuccess) return HLF_ERR_CUDA;
     if (cap == 0) return after_launch(h, HLF_OK, s);
-    return after_launch(h, hlf::launch_reduce_upto(enum_table(h), h->W, h->info_dev, cap, red_dev, s), s);
+    return after_launch(h, hlf::launch_reduce_upto(enum_table(h), h->W, dev_info(h), cap, red_dev, s), s);
 }
 
 hlf_status hlf_enumerate_store_dense(hlf_handle* h, uint64_t offset, uint64_t count, uint64_t* out_dev,

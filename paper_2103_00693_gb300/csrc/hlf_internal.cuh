@@ -103,10 +103,14 @@ struct FactorOut {
     uint64_t* table;   // [66][W]
     int32_t* info;     // [16]
     uint64_t* ptable;  // [66][W] or null: the paper-order table (see factor_impl.cuh)
-    int32_t* work;     // [kFactorWorkWords] device scratch of the n > 256 path (factor.cu), or null
+    int32_t* work;     // [kFactorWorkWords] device scratch, or null
 };
 
+// Device scratch of a factorisation: work[kFactorDevInfo ..] = status, rank as in
+// info, for kernels that read r (a read of the host-mapped words crosses the host
+// link); the rest serves the n > 256 path (factor.cu).
 constexpr int kFactorWorkWords = 64;
+constexpr int kFactorDevInfo = 24;
 
 // ---------------------------------------------------------------- launchers
 hlf_status launch_factor(const uint64_t* A, int n, int W, const FactorOut& o, cudaStream_t s);

@@ -1,5 +1,5 @@
 // Stage 2 for small instances without the rank on the host: the kernels read
-// r from the status word the factor kernel wrote.
+// r from the words the factor kernel left in the handle's device memory.
 //   store_upto_kernel   stores z(i) = z0 ^ XOR_{k in g(i)} B_k (Eq. 3 with
 //                       the Gray-code basis order) for every i < min(2^r, cap),
 //                       each straight from the definition. Meant for
@@ -22,18 +22,22 @@ __global__ void __launch_bounds__(kThreads) store_upto_kernel(const uint64_t* __
                                                               uint64_t* __restrict__ out)
 {
     __shared__ Table<W> t;
+    __shared__ SeedTable<W> st;
     __shared__ uint64_t s_count;
-    load_table<W>(t, table);
     if (threadIdx.x == 0) {
         const int32_t r = *reinterpret_cast<const volatile int32_t*>(info + 1);  // -1 after a fault
         s_count = r < 0 ? 0ull : (r >= 64 ? cap : (cap < (1ull << r) ? cap : (1ull << r)));
     }
+    load_table<W>(t, table);
     __syncthreads();
     const uint64_t count = s_count;
+    const int ntab = seed_tables_for(cap - 1);
+    build_seed_table<W>(st, t, ntab);
+    __syncthreads();
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t z[W];
-        seed<W>(t, i, z);
+        seed_lookup<W>(st, ntab, i, z);
         if (HLF_IN_BOUNDS(i, cap, kSiteUptoStore)) {
 #pragma unroll
             for (int w = 0; w < W; ++w) out[i * W + w] = z[w];
