@@ -40,11 +40,12 @@ namespace {
 // `parts` CTAs of blockDim.x threads, each thread walking `per` consecutive
 // indices that start at a multiple of 2^U, so that only the window's two ends
 // have partial Gray blocks. Items (window, part) are taken grid-stride. With
-// one part per window the CTA writes the result; otherwise it adds to it.
+// one part per window the CTA writes the result unless asked to add; otherwise it
+// adds to it.
 template <int W, int U, int T>
 __global__ void __launch_bounds__(T, min_ctas_for(W))
     reduce_kernel(const uint64_t* __restrict__ table, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
-                  uint32_t parts, uint64_t per, uint64_t runs, uint64_t align, int ntab,
+                  uint32_t parts, uint64_t per, uint64_t runs, uint64_t align, int ntab, bool add,
                   hlf_reduce* __restrict__ out)
 {
     __shared__ Table<W> t;
@@ -72,7 +73,7 @@ __global__ void __launch_bounds__(T, min_ctas_for(W))
         block_reduce<W, T>(cnt, acc);
         if (threadIdx.x != 0) continue;
         hlf_reduce& r = out[c];
-        if (parts == 1) {
+        if (parts == 1 && !add) {
             r.count = cnt;
             r.hsum = acc.hs;
 #pragma unroll
@@ -86,6 +87,175 @@ __global__ void __launch_bounds__(T, min_ctas_for(W))
                 if (f) atomicXor(reinterpret_cast<unsigned long long*>(&r.xor_fold[w]), (unsigned long long)f);
             }
         }
+    }
+}
+
+// ------------------------------------------------ large windows at W = 1
+// The reduce of one aligned region [base, base + 2^m) of indices, m >= kRegionMin.
+// Its solutions are z(base) ^ span(B_0 .. B_{m-1}) in whatever basis, so the walk may
+// choose one. In the L domain every vector has a low and a high 32-bit word, and at
+// least m - 32 dimensions of the span have a zero low word. With UH of these as the
+// innermost rows, the low word y_lo of 2^UH solutions in a row is the same, and with
+// it the low word of the hash's first product and most of the high one:
+//     y * M1 = y_lo * M1 + (y_hi * M1_lo << 32),
+// so a solution costs one 32-bit multiply-add where the product took a wide and two
+// narrow ones; the step XOR is one word; and since the product's low word p is fixed,
+// x ^= x >> 27 is a rotation of the high word by 5 and two masked XORs:
+//     lo' = (p ^ (p >> 27)) ^ (rot & ~31),  hi' = hi ^ (rot & 31).
+// 10 operations of the ALU pipe instead of 12, and 4 multiplies instead of 6.
+// 2^35 solutions (a rank-35 grid): 19.1 ms, 23.9 before; in a bare loop over 2^34,
+// UH = 4: 9.5 ms, 3: 9.5, 2: 9.8, the plain walk 12.5. Rows with a zero high word
+// inside gave 2%; the hash's last shift or its sum on the multiply pipe lost 1-10%.
+
+constexpr int kRegionMin = 33;
+
+// x = (lo, hi) behind the second shift: the last product and shift, added to hs.
+__device__ __forceinline__ void region_tail(uint32_t lo, uint32_t hi, uint64_t& hs)
+{
+    uint64_t y = (((uint64_t)hi << 32) | lo) * 0x94D049BB133111EBull;
+    hs += y ^ (y >> 31);
+}
+
+// 2^L solutions whose low words agree: p is the product's low word, kx = p ^ (p >> 27),
+// c the part of its high word that y_lo gives.
+template <int L, int UH>
+__device__ __forceinline__ void region_inner(uint32_t& yh, uint32_t kx, uint32_t c, const uint32_t (&BH)[UH],
+                                             uint64_t& hs)
+{
+    if constexpr (L == 0) {
+        const uint32_t h = yh * 0x1CE4E5B9u + c;
+        const uint32_t rot = __funnelshift_l(h, h, 5);
+        region_tail(kx ^ (rot & ~31u), h ^ (rot & 31u), hs);
+    } else {
+        region_inner<L - 1, UH>(yh, kx, c, BH, hs);
+        yh ^= BH[L - 1];
+        region_inner<L - 1, UH>(yh, kx, c, BH, hs);
+    }
+}
+
+// 2^(L + UH) solutions: the Gray walk over L general rows around the inner blocks.
+template <int L, int UH, int UL>
+__device__ __forceinline__ void region_block(uint32_t& yl, uint32_t& yh, const uint64_t (&BL)[UL],
+                                             const uint32_t (&BH)[UH], uint64_t& hs)
+{
+    if constexpr (L == 0) {
+        const uint64_t p = yl * 0xBF58476D1CE4E5B9ull;
+        const uint32_t pl = (uint32_t)p;
+        region_inner<UH, UH>(yh, pl ^ (pl >> 27), (uint32_t)(p >> 32), BH, hs);
+    } else {
+        region_block<L - 1, UH, UL>(yl, yh, BL, BH, hs);
+        yl ^= (uint32_t)BL[L - 1];
+        yh ^= (uint32_t)(BL[L - 1] >> 32);
+        region_block<L - 1, UH, UL>(yl, yh, BL, BH, hs);
+    }
+}
+
+constexpr int kRegionBlock = 6;  // log2 of the solutions unrolled
+
+// The run [j, j + len) of the region, whole blocks, from z(j) = y.
+template <int UH>
+__device__ __forceinline__ void region_run(const Table<1>& t, uint64_t j, uint64_t len, uint64_t y, uint64_t& hs)
+{
+    constexpr int UL = kRegionBlock - UH;
+    uint32_t BH[UH];
+    uint64_t BL[UL];
+#pragma unroll
+    for (int k = 0; k < UH; ++k) BH[k] = (uint32_t)(t.B[k][0] >> 32);
+#pragma unroll
+    for (int k = 0; k < UL; ++k) BL[k] = t.B[UH + k][0];
+    uint32_t yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
+    const uint64_t end = j + len;
+    for (;;) {
+        region_block<UL, UH, UL>(yl, yh, BL, BH, hs);
+        j += 1ull << kRegionBlock;
+        if (j >= end) break;
+        const uint64_t r = t.B[ctz64(j)][0];
+        yl ^= (uint32_t)r;
+        yh ^= (uint32_t)(r >> 32);
+    }
+}
+
+// Table in the L domain -> the region's: z0 = z(base), rows 0 .. m - 1 a basis of the
+// same span with the vectors of zero low word first, the others zero. Returns how
+// many those are. One warp reduces the low words as the elimination does (warp
+// maxima; lane l has rows l and l + 32): a row that becomes a pivot leaves the rest
+// and is a later row of the basis, what is left at the end has zero low words.
+__device__ int region_basis(Table<1>& t, uint64_t base, int m, int* s_u)
+{
+    const int lane = threadIdx.x & 31;
+    if (warp_uniform(threadIdx.x >> 5) == 0) {
+        const uint64_t g = base ^ (base >> 1);
+        const uint64_t seed_part = ((g >> lane) & 1u ? t.B[lane][0] : 0ull) ^
+                                   ((g >> (lane + 32)) & 1u ? t.B[lane + 32][0] : 0ull);
+        const uint64_t zb = (((uint64_t)__reduce_xor_sync(0xffffffffu, (uint32_t)(seed_part >> 32)) << 32) |
+                             __reduce_xor_sync(0xffffffffu, (uint32_t)seed_part)) ^
+                            t.z0[0];
+        uint64_t r0 = lane < m ? t.B[lane][0] : 0ull, r1 = lane + 32 < m ? t.B[lane + 32][0] : 0ull;
+        bool live0 = lane < m, live1 = lane + 32 < m;
+        __syncwarp();
+        int at = m;  // pivots fill the rows from the end
+        for (;;) {
+            const uint32_t q = __reduce_max_sync(0xffffffffu, max((uint32_t)r0, (uint32_t)r1));
+            if (!q) break;
+            // a row whose low word is q: the pivot. Any of them; lane `src`'s first.
+            const bool e0 = (uint32_t)r0 == q, e1 = (uint32_t)r1 == q;
+            const int src = __ffs(__ballot_sync(0xffffffffu, e0 || e1)) - 1;
+            const uint64_t p = __shfl_sync(0xffffffffu, e0 ? r0 : r1, src);
+            --at;
+            if (lane == src) {
+                t.B[at][0] = p;
+                if (e0) live0 = false, r0 = 0ull;
+                else live1 = false, r1 = 0ull;
+            }
+            const uint32_t top = 0x80000000u >> __clz(q);
+            if ((uint32_t)r0 & top) r0 ^= p;
+            if ((uint32_t)r1 & top) r1 ^= p;
+        }
+        const unsigned m0 = __ballot_sync(0xffffffffu, live0), m1 = __ballot_sync(0xffffffffu, live1);
+        const unsigned below = (1u << lane) - 1u;
+        if (live0) t.B[__popc(m0 & below)][0] = r0;
+        if (live1) t.B[__popc(m0) + __popc(m1 & below)][0] = r1;
+        for (int k = m + lane; k < kTableRows; k += 32) t.B[k][0] = 0ull;
+        if (lane == 0) {
+            t.z0[0] = zb;
+            *s_u = at;
+        }
+    }
+    __syncthreads();
+    return *s_u;
+}
+
+__global__ void __launch_bounds__(1024, 1) reduce_region_kernel(const uint64_t* __restrict__ table, uint64_t base,
+                                                                int m, uint64_t per, hlf_reduce* __restrict__ out)
+{
+    __shared__ Table<1> t;
+    __shared__ SeedTable<1> st;
+    __shared__ int s_u;
+    load_table_hash_domain<1, 2>(t, table);
+    __syncthreads();
+    const int u = region_basis(t, base, m, &s_u);
+    const int ntab = (m + 3) / 4;
+    build_seed_table<1>(st, t, ntab);
+    __syncthreads();
+    const uint64_t size = 1ull << m;
+    const uint64_t j = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * per;
+    Acc<1> acc;
+    acc.zero();  // the fold of a whole region is zero
+    uint64_t cnt = 0;
+    if (j < size) {
+        cnt = min(per, size - j);
+        uint64_t z[1];
+        seed_lookup<1>(st, ntab, j, z);
+        if (u >= 4) region_run<4>(t, j, cnt, z[0], acc.hs);
+        else if (u == 3) region_run<3>(t, j, cnt, z[0], acc.hs);
+        else if (u == 2) region_run<2>(t, j, cnt, z[0], acc.hs);
+        else if (u == 1) region_run<1>(t, j, cnt, z[0], acc.hs);
+        else reduce_run_from<1, kRegionBlock>(t, false, j, cnt, z, acc);
+    }
+    block_reduce<1, 1024>(cnt, acc);
+    if (threadIdx.x == 0 && cnt) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(&out->count), (unsigned long long)cnt);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&out->hsum), (unsigned long long)acc.hs);
     }
 }
 
@@ -253,37 +423,75 @@ ReduceShape reduce_shape(uint64_t chunk, uint64_t n_chunks)
     return sh;
 }
 
+// add: *out is a sum in progress (one window).
 template <int W, int U>
 hlf_status launch_reduce_u(const uint64_t* table, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
-                           hlf_reduce* out, cudaStream_t s)
+                           hlf_reduce* out, cudaStream_t s, bool add = false)
 {
     constexpr int T = reduce_threads(W);
     const ReduceShape sh = reduce_shape<W, U, T>(chunk, n_chunks);
-    if (sh.parts > 1 && cudaMemsetAsync(out, 0, sizeof(hlf_reduce) * n_chunks, s) != cudaSuccess)
+    if (sh.parts > 1 && !add && cudaMemsetAsync(out, 0, sizeof(hlf_reduce) * n_chunks, s) != cudaSuccess)
         return HLF_ERR_CUDA;
     const int ntab = seed_tables_for(offset + (chunk * n_chunks - 1));
     reduce_kernel<W, U, T><<<sh.blocks, sh.threads, 0, s>>>(table, offset, chunk, n_chunks, sh.parts, sh.per, sh.runs,
-                                                           sh.align, ntab, out);
+                                                           sh.align, ntab, add, out);
     return cudaGetLastError() == cudaSuccess ? HLF_OK : HLF_ERR_CUDA;
 }
 
 // W = 1 has two unrolls: 2^6 solutions per Gray block where every thread of a
 // full wave has at least 16 blocks, else 2^3, whose finer cut balances and
 // fills the SMs better than the deeper unroll saves.
+hlf_status launch_reduce_1(const uint64_t* table, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
+                           hlf_reduce* out, cudaStream_t s, bool add)
+{
+    const uint64_t wave = (uint64_t)sm_count() * min_ctas_for(1) * reduce_threads(1);
+    if (chunk * n_chunks < wave * 1024) return launch_reduce_u<1, 3>(table, offset, chunk, n_chunks, out, s, add);
+    return launch_reduce_u<1, reduce_unroll(1)>(table, offset, chunk, n_chunks, out, s, add);
+}
+
+// One window of at least 2^kRegionMin solutions at W = 1: its aligned regions of that
+// size and more, the largest that fit (at most two of each size), and what lies
+// before and after them.
+hlf_status launch_reduce_regions(const uint64_t* table, uint64_t offset, uint64_t count, hlf_reduce* out,
+                                 cudaStream_t s)
+{
+    if (cudaMemsetAsync(out, 0, sizeof(hlf_reduce), s) != cudaSuccess) return HLF_ERR_CUDA;
+    const uint64_t threads = (uint64_t)sm_count() * 1024;
+    for (uint64_t a = offset, left = count; left;) {
+        int m = 63;
+        while (m >= kRegionMin && ((1ull << m) > left || (a & ((1ull << m) - 1)))) --m;
+        uint64_t size;
+        if (m >= kRegionMin) {
+            size = 1ull << m;
+            uint64_t per = (size + threads - 1) / threads;
+            per = (per + (1ull << kRegionBlock) - 1) & ~((1ull << kRegionBlock) - 1);
+            reduce_region_kernel<<<(unsigned)((size + per * 1024 - 1) / (per * 1024)), 1024, 0, s>>>(table, a, m, per,
+                                                                                                  out);
+            if (cudaGetLastError() != cudaSuccess) return HLF_ERR_CUDA;
+        } else {  // up to the next multiple of 2^kRegionMin, or the end
+            size = (1ull << kRegionMin) - (a & ((1ull << kRegionMin) - 1));
+            if (size > left) size = left;
+            const hlf_status st = launch_reduce_1(table, a, size, 1, out, s, true);
+            if (st != HLF_OK) return st;
+        }
+        a += size;
+        left -= size;
+    }
+    return HLF_OK;
+}
+
 template <int W>
 hlf_status launch_reduce_w(const uint64_t* table, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
                            hlf_reduce* out, cudaStream_t s)
 {
     if constexpr (W == 1) {
-        const uint64_t wave = (uint64_t)sm_count() * min_ctas_for(1) * reduce_threads(1);
-        if (chunk * n_chunks < wave * 1024) return launch_reduce_u<1, 3>(table, offset, chunk, n_chunks, out, s);
+        if (n_chunks == 1 && chunk >= 1ull << kRegionMin) return launch_reduce_regions(table, offset, chunk, out, s);
+        return launch_reduce_1(table, offset, chunk, n_chunks, out, s, false);
+    } else {
+        return launch_reduce_u<W, reduce_unroll(W)>(table, offset, chunk, n_chunks, out, s);
     }
-    return launch_reduce_u<W, reduce_unroll(W)>(table, offset, chunk, n_chunks, out, s);
 }
 
-// One wave of warps, each with consecutive groups; short windows give a warp one
-// group and spread the warps over the SMs (2^14 solutions of two words on one CTA
-// took 13 us, a group a warp on 64 CTAs takes 4).
 template <int W>
 hlf_status launch_store_w(const uint64_t* table, uint64_t offset, uint64_t count, uint64_t* out,
                           cudaStream_t s)

@@ -121,12 +121,6 @@ __device__ __forceinline__ uint64_t* factor_rows(unsigned char* smem)
     return reinterpret_cast<uint64_t*>(smem + (sizeof(FactorSmem<W, MAXN>) + 15) / 16 * 16);
 }
 
-// A value that is the same in every lane of the warp, in a form that lets the
-// compiler know it: a branch on it keeps the warp converged. Behind a branch that
-// might split the warp every warp-wide operation is preceded by a
-// reconvergence, which doubled the time of the searches below.
-__device__ __forceinline__ int warp_uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
-
 // The warps of an elimination (W > 1). An SM's four schedulers take a CTA's warps
 // by their number mod 4. The searching warp is a serial chain of instructions, so
 // it has a scheduler to itself: it is warp 3, the row warps are those whose number

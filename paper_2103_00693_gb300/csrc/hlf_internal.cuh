@@ -155,6 +155,10 @@ __device__ __forceinline__ uint64_t mix64(uint64_t x)
     return x;
 }
 
+// A value that is the same in every lane of the warp, in a form that lets the
+// compiler know it: a branch on it keeps the warp converged.
+__device__ __forceinline__ int warp_uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+
 // Index of the lowest set bit; 64 for x == 0 (so the zero row 64 is used).
 __device__ __forceinline__ int ctz64(uint64_t x) { return __clzll(__brevll(x)); }
 
