@@ -125,7 +125,17 @@ __device__ void batch_reduce_chunk(const BatchArgs& a, int b, uint64_t first, ui
     constexpr uint64_t kBlk = 1ull << U;
     Table<W>& t = *reinterpret_cast<Table<W>*>(smem);
     SeedTable<W>& st = *reinterpret_cast<SeedTable<W>*>(smem + sizeof(Table<W>));
-    const bool mixed = __syncthreads_or(load_table_hash_domain<W, U>(t, a.tables + (size_t)b * kTableSlot));
+    bool mixed = __syncthreads_or(load_table_hash_domain<W, U>(t, a.tables + (size_t)b * kTableSlot));
+    // A chunk that is an aligned region (all but an instance's last, where cap is no
+    // power of two) is walked over a basis whose first rows step word 0 only, unless the
+    // table's own do: 1024 grids 1973 -> 1907 us.
+    if constexpr (W > 1) {
+        if (mixed && (len & (len - 1)) == 0 && (first & (len - 1)) == 0 && len > kBlk && len <= 1ull << 32) {
+            __shared__ int s_low;
+            mixed = low_basis<W>(t, first, 63 - __clzll((long long)len), &s_low) < U;
+            first = 0;
+        }
+    }
     const int ntab = seed_tables_for(first + len - 1);
     build_seed_table<W>(st, t, ntab);
     __syncthreads();

@@ -273,6 +273,65 @@ __device__ __forceinline__ void reduce_run_from(const Table<W>& t, bool mixed, u
     }
 }
 
+// Table in the L domain -> the table of an aligned region [base, base + 2^m) of
+// indices, 0 < m <= 32, whose solutions are z(base) ^ span(B_0 .. B_{m-1}) in any
+// basis: z0 = z(base), rows 0 .. m - 1 a basis with the vectors of zero words past
+// word 0 first. Returns how many those are. The region's index counts from base.
+// One warp reduces the later words, lane l holding row l: a warp maximum names a
+// pivot, which leaves the rest and becomes a later row of the basis; what is left at
+// the end has word 0 only. Called by the whole CTA.
+template <int W>
+__device__ int low_basis(Table<W>& t, uint64_t base, int m, int* s_low)
+{
+    const int lane = threadIdx.x & 31;
+    if (warp_uniform(threadIdx.x >> 5) == 0) {
+        const uint64_t g = base ^ (base >> 1);
+        const bool lo = (g >> lane) & 1u, hi = (g >> (lane + 32)) & 1u;
+        uint64_t r[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const uint64_t a = (lo ? t.B[lane][w] : 0ull) ^ (hi ? t.B[lane + 32][w] : 0ull);
+            const uint32_t al = __reduce_xor_sync(0xffffffffu, (uint32_t)a);
+            const uint32_t ah = __reduce_xor_sync(0xffffffffu, (uint32_t)(a >> 32));
+            if (lane == 0) t.z0[w] ^= ((uint64_t)ah << 32) | al;
+            r[w] = lane < m ? t.B[lane][w] : 0ull;
+        }
+        bool live = lane < m;
+        __syncwarp();
+        int at = m;  // pivots fill the rows from the end
+#pragma unroll
+        for (int w = 1; w < W; ++w) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                for (;;) {
+                    const uint32_t v = (uint32_t)(r[w] >> (32 * h));
+                    const uint32_t q = __reduce_max_sync(0xffffffffu, v);
+                    if (!q) break;
+                    const int src = __ffs(__ballot_sync(0xffffffffu, v == q)) - 1;
+                    const bool has = v & (0x80000000u >> __clz(q));
+                    --at;
+#pragma unroll
+                    for (int x = 0; x < W; ++x) {
+                        const uint64_t p = __shfl_sync(0xffffffffu, r[x], src);
+                        if (lane == src) t.B[at][x] = p;
+                        r[x] ^= has ? p : 0ull;  // the pivot's own row becomes zero
+                    }
+                    if (lane == src) live = false;
+                }
+            }
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, live);
+        if (live) {
+            const int k = __popc(mask & ((1u << lane) - 1u));
+#pragma unroll
+            for (int x = 0; x < W; ++x) t.B[k][x] = x ? 0ull : r[0];
+        }
+        if (lane == 0) *s_low = at;
+    }
+    __syncthreads();
+    return *s_low;
+}
+
 // Block-wide (count, hsum, fold) reduction over a CTA of THREADS threads;
 // the result is valid in thread 0.
 template <int W, int THREADS = kThreads>
