@@ -342,8 +342,10 @@ __global__ void __launch_bounds__(kD2Threads) dense2_kernel(const uint64_t* __re
     uint64_t zA[W], zB[W];
     const uint64_t iA = pl.offset + 64 * k0 + tA;
     uint64_t HA = iA >> 6, HB = (iA + 1) >> 6;
-    seed<W>(t, iA, zA);
-    seed<W>(t, iA + 1, zB);
+    seed_near<W>([&](int r) { return r == kTableZ0Row ? t.z0 : t.B[r]; }, pl.offset + 64 * k0, iA, lane, zA);
+    const uint64_t* rB = t.B[ctz64(iA + 1)];
+#pragma unroll
+    for (int w = 0; w < W; ++w) zB[w] = zA[w] ^ rB[w];
 
     // P consecutive groups share a staging buffer and leave in one store
     for (uint64_t k = k0;;) {
@@ -768,7 +770,12 @@ hlf_status launch_dense2(const uint64_t* table, int n, uint64_t offset, uint64_t
 hlf_status launch_store_dense(const uint64_t* table, int n, uint64_t offset, uint64_t count, uint64_t* out,
                               cudaStream_t s)
 {
-    if (n == 64) return launch_store(table, 1, offset, count, out, s);  // one whole word per solution
+    // Whole words per solution: the stream is the packed store. On 1 GB windows it writes
+    // 6.4 TB/s at n = 512 and 6.2 at 1024, where placing words 64 n bits apart collides
+    // in shared memory (2.2), and 6.2-6.3 against 6.0-6.1 at n = 128 and 256; 16411
+    // solutions take 4-6 us instead of 8-16. It wants 16 bytes at W > 1.
+    if (n == 64 || (n % 64 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0))
+        return launch_store(table, n / 64, offset, count, out, s);
     if (n < 64) {
         const int m = 64 / (n & -n);  // 64 / gcd(n, 64)
         const int M = m < 16 ? 16 : m;

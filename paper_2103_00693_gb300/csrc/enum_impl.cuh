@@ -497,6 +497,56 @@ __device__ __forceinline__ void seed_group(Row row, uint64_t h, int lane, uint64
     }
 }
 
+// z(i) for lanes whose indices lie in [base, base + 64), base the same in all of them:
+// i >> 6 is one of two consecutive values, so all but the last six rows and the step
+// between the two are shared (as in seed_group).
+template <int W, typename Row>
+__device__ __forceinline__ void seed_near(Row row, uint64_t base, uint64_t i, int lane, uint64_t (&z)[W])
+{
+    const uint64_t H = base >> 6;
+    const uint64_t g = ((H ^ (H >> 1)) << 6) ^ ((H & 1) << 5);
+    const bool lo = (g >> lane) & 1u, hi = (g >> (lane + 32)) & 1u;
+    const bool next = (i >> 6) != H;
+    const int gt = (int)(i & 63) ^ ((int)(i & 63) >> 1);
+    const int j = ctz64(H + 1);  // at most 58
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        const uint64_t a = (lo ? row(lane)[w] : 0ull) ^ (hi ? row(lane + 32)[w] : 0ull);
+        z[w] = ((uint64_t)__reduce_xor_sync(0xffffffffu, (uint32_t)(a >> 32)) << 32) |
+               __reduce_xor_sync(0xffffffffu, (uint32_t)a);
+        z[w] ^= row(kTableZ0Row)[w] ^ (next ? row(5)[w] ^ row(6 + j)[w] : 0ull);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const bool in = (gt >> k) & 1;
+#pragma unroll
+        for (int w = 0; w < W; ++w) z[w] ^= in ? row(k)[w] : 0ull;
+    }
+}
+
+// The ragged ends of a window, 32 indices a warp: share `u` of ragged_shares(g).
+__host__ __device__ inline uint64_t ragged_shares(const GroupPlan& g)
+{
+    return (g.n_head + 31) / 32 + (g.n_tail + 31) / 32;
+}
+template <int W, typename Row, typename Check>
+__device__ __forceinline__ void store_ragged(Row row, const GroupPlan& g, uint64_t offset, uint64_t u, uint64_t* out,
+                                             int lane, Check ok)
+{
+    const uint64_t heads = (g.n_head + 31) / 32;
+    const bool head = u < heads;
+    const uint64_t at = 32 * (head ? u : u - heads);
+    const uint64_t left = (head ? g.n_head : g.n_tail) - at;
+    const uint64_t base = (head ? offset : g.tail_first) + at;
+    const uint64_t i = base + lane;
+    uint64_t z[W];
+    seed_near<W>(row, base, i, lane, z);
+    if (lane < left && ok(i, 1)) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) out[(i - offset) * W + w] = z[w];
+    }
+}
+
 // Groups [h, h1) of a window, h < h1, by one warp from the lanes' seeds: `dst` is the
 // output less offset * W words, `step(j)` points to C_j, `b0` is B_0's word (W = 1),
 // `stage` holds stage_words<W>() words of the warp (W > 1). W = 1 needs dst + odd on

@@ -262,7 +262,8 @@ __global__ void __launch_bounds__(1024, 1) reduce_region_kernel(const uint64_t* 
 struct StorePlan {
     uint64_t offset, count;
     GroupPlan g;
-    uint64_t per_warp;  // groups per warp
+    uint64_t warps;     // with groups, per_warp each (the last may have fewer)
+    uint64_t per_warp;
 };
 
 template <int W>
@@ -282,30 +283,20 @@ __global__ void __launch_bounds__(kThreads) store_kernel(const uint64_t* __restr
     }
     __syncthreads();
 
-    const uint64_t gt = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    // ragged head and tail, one index per thread, from the definition
-    if (gt < pl.g.n_head + pl.g.n_tail) {
-        const uint64_t i = gt < pl.g.n_head ? pl.offset + gt : pl.g.tail_first + (gt - pl.g.n_head);
-        uint64_t z[W];
-        seed<W>(t, i, z);
-        if (HLF_IN_BOUNDS(i - pl.offset, pl.count, kSiteStore)) {
-#pragma unroll
-            for (int w = 0; w < W; ++w) out[(i - pl.offset) * W + w] = z[w];
-        }
-    }
-    __syncwarp();
-
-    const uint64_t wg = gt >> 5;
+    const uint64_t wg = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    auto row = [&](int k) { return k == kTableZ0Row ? t.z0 : t.B[k]; };
+    auto ok = [&](uint64_t i, uint64_t len) { return HLF_RANGE_IN_BOUNDS(i - pl.offset, len, pl.count, kSiteStore); };
+    if (wg >= pl.warps) {  // the last warps have the ragged ends
+        if (wg - pl.warps < ragged_shares(pl.g)) store_ragged<W>(row, pl.g, pl.offset, wg - pl.warps, out, lane, ok);
+        return;
+    }
     const uint64_t h0 = pl.g.h_first + wg * pl.per_warp;
-    if (wg * pl.per_warp >= pl.g.h_end - pl.g.h_first) return;
     const uint64_t h1 = min(h0 + pl.per_warp, pl.g.h_end);
     uint64_t z[W];
-    seed_group<W>([&](int k) { return k == kTableZ0Row ? t.z0 : t.B[k]; }, h0, lane, z);
-    store_groups<W>(
-        z, h0, h1, pl.g.odd, t.B[0][0], out - pl.offset * W, s_stage + (threadIdx.x >> 5) * stage_words<W>(), lane,
-        [&](int j) { return s_C[j]; },
-        [&](uint64_t i, uint64_t len) { return HLF_RANGE_IN_BOUNDS(i - pl.offset, len, pl.count, kSiteStore); });
+    seed_group<W>(row, h0, lane, z);
+    store_groups<W>(z, h0, h1, pl.g.odd, t.B[0][0], out - pl.offset * W,
+                    s_stage + (threadIdx.x >> 5) * stage_words<W>(), lane, [&](int j) { return s_C[j]; }, ok);
 }
 
 // ----------------------------------------------------------------- sample
@@ -517,13 +508,9 @@ hlf_status launch_store_w(const uint64_t* table, uint64_t offset, uint64_t count
     }
     const uint64_t sms = (uint64_t)sm_count();
     const uint64_t max_warps = sms * fit[dev] * (kThreads / 32);
-    uint64_t warps = groups < max_warps ? groups : max_warps;
-    if (warps == 0) warps = 1;
-    pl.per_warp = groups ? (groups + warps - 1) / warps : 1;
-    if (groups) warps = (groups + pl.per_warp - 1) / pl.per_warp;
-    const uint64_t ragged = pl.g.n_head + pl.g.n_tail;
-    uint64_t threads = warps * 32;
-    if (threads < ragged) threads = ragged;
+    pl.per_warp = groups ? (groups + max_warps - 1) / max_warps : 1;
+    pl.warps = (groups + pl.per_warp - 1) / pl.per_warp;
+    const uint64_t threads = 32 * (pl.warps + ragged_shares(pl.g));
     uint64_t bd = (threads / sms + 31) / 32 * 32;
     bd = bd < 64 ? 64 : (bd > kThreads ? kThreads : bd);
     const unsigned blocks = (unsigned)((threads + bd - 1) / bd);

@@ -3,10 +3,9 @@
 // stage-2 materialisation of hlf_enumerate_store (Section 2, Fig. 1(c)); the
 // batching only schedules them together.
 //
-// The host cuts every window into tasks of about 4 KB of output: task 0 of a window
-// writes its ragged head and tail (the indices outside its groups, seeded one by
-// one from the definition), the others cover task_groups(W) groups of consecutive
-// indices each. A warp takes an equal run of tasks, finds its first window by binary
+// The host cuts every window into tasks of about 4 KB of output: the first of a
+// window write its ragged ends (the indices outside its groups), 32 indices each,
+// the others cover task_groups(W) groups of consecutive indices each. A warp takes an equal run of tasks, finds its first window by binary
 // search over the task prefix sums, and stores the groups of each window in the run
 // in one walk (store_groups), so that it seeds itself once a window: a seed is one
 // round of loads, every lane bringing two rows, and the window's first step rows are
@@ -37,50 +36,27 @@ struct WinDesc {
 
 constexpr int kWarpWords = stage_words<HLF_MAX_W>() + kTaskRows * HLF_MAX_W;  // shared words per warp
 
-template <int W>
-__device__ __forceinline__ void seed_g(const uint64_t* __restrict__ tab, uint64_t i, uint64_t (&z)[W])
-{
-    uint64_t g = i ^ (i >> 1);
-#pragma unroll
-    for (int w = 0; w < W; ++w) z[w] = __ldg(tab + kTableZ0Row * W + w);
-    while (g) {
-        const int k = __ffsll((long long)g) - 1;
-        g &= g - 1;
-#pragma unroll
-        for (int w = 0; w < W; ++w) z[w] ^= __ldg(tab + k * W + w);
-    }
-}
-
 // Tasks [u, u1) of window d by one warp.
 template <int W>
 __device__ void many_tasks(const WinDesc& d, uint64_t u, uint64_t u1, int lane, uint64_t* stage)
 {
     constexpr int M = Groups<W>::kLog2;
-    const uint64_t ragged = d.g.n_head + d.g.n_tail;
-    if (ragged) {
-        if (u == 0)
-            for (uint64_t e = lane; e < ragged; e += 32) {
-                const uint64_t i = e < d.g.n_head ? d.offset + e : d.g.tail_first + (e - d.g.n_head);
-                uint64_t z[W];
-                seed_g<W>(d.table, i, z);
-                if (HLF_IN_BOUNDS(i - d.offset, d.count, kSiteManyStore)) {
-#pragma unroll
-                    for (int w = 0; w < W; ++w) d.out[(i - d.offset) * W + w] = z[w];
-                }
-            }
-        __syncwarp();
-        u -= u != 0;  // task t > 0 covers the groups of index t - 1
-        --u1;
-    }
+    const uint64_t* tab = d.table;
+    auto row = [&](int k) { return tab + k * W; };
+    auto ok = [&](uint64_t i, uint64_t len) { return HLF_RANGE_IN_BOUNDS(i - d.offset, len, d.count, kSiteManyStore); };
+    const uint64_t ragged = ragged_shares(d.g);  // the first tasks
+    for (; u < min(ragged, u1); ++u) store_ragged<W>(row, d.g, d.offset, u, d.out, lane, ok);
+    if (u >= u1) return;
+    u -= ragged;
+    u1 -= ragged;
     const uint64_t h0 = d.g.h_first + u * task_groups(W);
     const uint64_t h1 = min(d.g.h_first + u1 * task_groups(W), d.g.h_end);
     if (h0 >= h1) return;
     uint64_t* C = stage + stage_words<HLF_MAX_W>();  // [kTaskRows][W]
-    const uint64_t* tab = d.table;
     for (int e = lane; e < kTaskRows * W; e += 32)
         C[e] = __ldg(tab + (M - 1) * W + e % W) ^ __ldg(tab + M * W + e);
     uint64_t z[W];
-    seed_group<W>([&](int k) { return tab + k * W; }, h0, lane, z);
+    seed_group<W>(row, h0, lane, z);
     __syncwarp();
     uint64_t rare[W];  // a step row that is not staged
     store_groups<W>(
@@ -91,7 +67,7 @@ __device__ void many_tasks(const WinDesc& d, uint64_t u, uint64_t u1, int lane, 
             for (int w = 0; w < W; ++w) rare[w] = __ldg(tab + (M - 1) * W + w) ^ __ldg(tab + (M + j) * W + w);
             return rare;
         },
-        [&](uint64_t i, uint64_t len) { return HLF_RANGE_IN_BOUNDS(i - d.offset, len, d.count, kSiteManyStore); });
+        ok);
     __syncwarp();  // the staged rows are rewritten for the next window
 }
 
@@ -144,7 +120,7 @@ void plan_window(WinDesc& d, uint32_t W)
     d.g = plan_groups(d.offset, d.count, G, W == 1 ? d.offset & 1 : 0);
     d.W = W;
     const uint64_t tg = task_groups(W);
-    d.ntasks = (uint32_t)((d.g.n_head + d.g.n_tail ? 1 : 0) + (d.g.h_end - d.g.h_first + tg - 1) / tg);
+    d.ntasks = (uint32_t)(ragged_shares(d.g) + (d.g.h_end - d.g.h_first + tg - 1) / tg);
 }
 
 }  // namespace
