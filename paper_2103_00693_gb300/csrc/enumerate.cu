@@ -362,8 +362,8 @@ struct ReduceShape {
 // costs a few tens of solutions (kSeedCost), so short runs are worth it
 // whenever they fill idle SMs. One window: one CTA if that holds them all (the
 // result then needs no clearing), else all of them, up to one wave, in CTAs no
-// larger than spreading them over every SM takes. Several windows: the largest
-// CTA a window fills, and the cut whose waves cost least.
+// larger than spreading them over every SM takes. Several windows: the CTA size and
+// the cut whose waves cost least.
 // With runs of at least 2048 indices and one CTA per window instead, 2^20
 // four-word solutions took 694 us on one SM (now 12.4, two launches and the
 // host's call among it), and 64 windows of 2^24 at W = 1 took 2.16 ms on 64
@@ -385,19 +385,24 @@ ReduceShape reduce_shape(uint64_t chunk, uint64_t n_chunks)
         sh.threads = (unsigned)bd;
         sh.parts = (uint32_t)((want + bd - 1) / bd);
     } else {
-        uint64_t bd = T;
-        while (bd > 64 && bd > runs) bd /= 2;
-        sh.threads = (unsigned)bd;
-        const uint64_t slots = sms * (room / bd);
+        // CTAs of T threads down to 64, 1 to 64 of them a window: the fewest steps of
+        // the busiest SM. Smaller CTAs only where that saves 1/16: each builds its own
+        // tables (64 windows of 2^24 in CTAs of 64 threads 813 us, of 1024 792, though
+        // the former fill the wave 3% better; 64 of 1239596 78 us against 82).
         uint64_t best = ~0ull;
-        for (uint64_t k = 1; k <= 64 && (k == 1 || (k - 1) * bd < runs); ++k) {
-            const uint64_t waves = (n_chunks * k + slots - 1) / slots;
-            const uint64_t cost = waves * (kSeedCost + (chunk + k * bd - 1) / (k * bd));
-            if (cost < best) {
-                best = cost;
-                sh.parts = (uint32_t)k;
+        for (uint64_t bd = T; bd >= 64; bd /= 2) {
+            const uint64_t slots = sms * (room / bd);
+            const uint64_t least = best - best / 16;
+            for (uint64_t k = 1; k <= 64 && (k == 1 || (k - 1) * bd < runs); ++k) {
+                const uint64_t waves = (n_chunks * k + slots - 1) / slots;
+                const uint64_t cost = waves * (kSeedCost + (((chunk - 1) / (k * bd)) | ((1ull << U) - 1)) + 1);
+                if (cost < best && (bd == T || cost < least)) {
+                    best = cost;
+                    sh.parts = (uint32_t)k;
+                    sh.threads = (unsigned)bd;
+                }
+                if (n_chunks > (~0ull >> 8)) break;  // a window each is enough
             }
-            if (n_chunks > (~0ull >> 8)) break;  // a window each is enough
         }
     }
     want = (uint64_t)sh.parts * sh.threads;
