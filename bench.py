@@ -50,6 +50,13 @@ ISSUE_LANES_PER_SM_CLK = 128  # 4 schedulers x 32 lanes
 # ALU pipe executes (64 lanes per clock per SM): the step XOR 2, the two
 # xor-shifts 8 and the 64-bit add 2. The multiplies run on the FMA pipe.
 ALU_PIPE_OPS_PER_SOLUTION_W1 = 12
+# The headline reduce (W = 1, an aligned region of at least 2^33 solutions) is walked
+# over a basis whose inner rows leave the low word alone: step XOR 1, the high word's
+# multiply-add 1, the second shift 3 (a rotation and two masked XORs), the last
+# multiply 3, the last shift 4 and the add 2 are 14 operations, 10 of them on the ALU
+# pipe; what a block of 8 or 16 solutions shares is not counted.
+REGION_OPS_PER_SOLUTION = 14
+REGION_ALU_OPS_PER_SOLUTION = 10
 ALU_PIPE_LANES_PER_SM_CLK = 64
 PROBE_ITERS = 1 << 14
 STORE_LOG2 = 30
@@ -63,13 +70,13 @@ SAMPLE_SEED = 99
 # sources change, the figure no longer describes the kernel and the line
 # reports null.
 KERNEL_SOURCES = {
-    "reduce_kernel<1,6,1024>": ["enumerate.cu", "enum_impl.cuh", "hlf_internal.cuh"],
-    "store_kernel<1,2>": ["enumerate.cu", "enum_impl.cuh", "hlf_internal.cuh"],
+    "reduce_region_kernel": ["enumerate.cu", "enum_impl.cuh", "hlf_internal.cuh"],
+    "store_kernel<1>": ["enumerate.cu", "enum_impl.cuh", "hlf_internal.cuh"],
     "dense1_kernel<16,1,1>": ["dense.cu", "enum_impl.cuh", "hlf_internal.cuh"],
 }
 TRAFFIC = {  # kernel -> per-launch DRAM bytes (read + write) and the source digest at capture
-    "reduce_kernel<1,6,1024>": {"bytes": 541440 + 1536, "sources": "0b975b98a6be7595"},
-    "store_kernel<1,2>": {"bytes": 244992 + 8525198848, "sources": "0b975b98a6be7595"},
+    "reduce_region_kernel": {"bytes": 541440 + 1536, "sources": "0b975b98a6be7595"},
+    "store_kernel<1>": {"bytes": 244992 + 8525198848, "sources": "0b975b98a6be7595"},
     "dense1_kernel<16,1,1>": {"bytes": 467200 + 4767411200, "sources": "2a92c04830996b04"},
 }
 
@@ -112,7 +119,8 @@ def parse():
 
 
 def ops_per_solution(W: int) -> int:
-    """The reduce's minimal 32-bit integer operations per solution of W words."""
+    """32-bit integer operations per solution of W words, each word walked as it is
+    (the reference mix; walk_ops has the reduce's own)."""
     return OPS_PER_SOLUTION_W1 + 22 * (W - 1)
 
 
@@ -122,6 +130,24 @@ def alu_pipe_ops_per_solution(W: int) -> int:
     three xor-shifts of its SplitMix64 round 12 (the round's two multiplies
     run on the FMA pipe)."""
     return ALU_PIPE_OPS_PER_SOLUTION_W1 + 16 * (W - 1)
+
+
+def walk_ops(W: int) -> int:
+    """The operations per solution of the walk as the general reduce runs it: every
+    word is kept behind the finalizer's linear first layer, so a later word joins the
+    chained hash's layer as a third operand of its XORs: 20 a word beyond the first."""
+    return OPS_PER_SOLUTION_W1 + 20 * (W - 1)
+
+
+def walk_alu_ops(W: int) -> int:
+    return ALU_PIPE_OPS_PER_SOLUTION_W1 + 14 * (W - 1)
+
+
+def headline_reduce(W: int, count: int):
+    """(kernel, operations, ALU-pipe operations per solution) of a reduce of `count`."""
+    if W == 1 and count >= 1 << 33:
+        return "reduce_region_kernel", REGION_OPS_PER_SOLUTION, REGION_ALU_OPS_PER_SOLUTION
+    return f"reduce_kernel<{W}>", walk_ops(W), walk_alu_ops(W)
 
 
 def alu_pipe_peak(dev=None):
@@ -441,8 +467,8 @@ def run_hlf(args, world, rank, local):
     pk = peaks()
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     alu_peak = sms * ISSUE_LANES_PER_SM_CLK * pk["sm_max_mhz"] * 1e6 / 1e12  # Tops/s
-    ops = total * ops_per_solution(W)
-    achieved = ops / (reduce_ms / 1e3) / 1e12
+    red_kernel, red_ops, red_alu = headline_reduce(W, total)
+    achieved = total * red_ops / (reduce_ms / 1e3) / 1e12
     store_bytes = store_n * W * 8
     store_gbs = store_bytes / (store_ms / 1e3) / 1e9
 
@@ -451,24 +477,24 @@ def run_hlf(args, world, rank, local):
             "scaling": "weak", "vs_baseline": None, "dtype": "u64", "data": "synthetic",
             "config": workload_config(r, total, store_n),
             "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "Tops/s",
-                         "frac": achieved / alu_peak, "traffic": traffic("reduce_kernel<1,6,1024>"),
-                         "kernel": "reduce_kernel<1,6,1024>",
+                         "frac": achieved / alu_peak, "traffic": traffic(red_kernel),
+                         "kernel": red_kernel,
                          "ms_per_launch": reduce_ms,
                          "peak_basis": f"{sms} SMs x {ISSUE_LANES_PER_SM_CLK} int32 lanes/clk x "
                                        f"{pk['sm_max_mhz']:.0f} MHz (issue limit)",
-                         "ops_per_solution": ops_per_solution(W)},
+                         "ops_per_solution": red_ops},
             "roofline_alu_pipe": {
                 "bound": "alu_pipe",
-                "achieved": total * ALU_PIPE_OPS_PER_SOLUTION_W1 / (reduce_ms / 1e3) / 1e12,
+                "achieved": total * red_alu / (reduce_ms / 1e3) / 1e12,
                 "peak": sms * ALU_PIPE_LANES_PER_SM_CLK * pk["sm_max_mhz"] * 1e6 / 1e12, "unit": "Tops/s",
-                "frac": (total * ALU_PIPE_OPS_PER_SOLUTION_W1 / (reduce_ms / 1e3))
+                "frac": (total * red_alu / (reduce_ms / 1e3))
                         / (sms * ALU_PIPE_LANES_PER_SM_CLK * pk["sm_max_mhz"] * 1e6),
-                "kernel": "reduce_kernel<1,6,1024>", "ops_per_solution": ALU_PIPE_OPS_PER_SOLUTION_W1,
+                "kernel": red_kernel, "ops_per_solution": red_alu,
                 "peak_basis": f"{sms} SMs x {ALU_PIPE_LANES_PER_SM_CLK} ALU-pipe lanes/clk x "
                               f"{pk['sm_max_mhz']:.0f} MHz (the pipe that binds: W = 1 only)"} if W == 1 else None,
             "roofline_store": {"bound": "hbm", "achieved": store_gbs, "peak": pk["hbm_gbs"], "unit": "GB/s",
-                               "frac": store_gbs / pk["hbm_gbs"], "traffic": traffic("store_kernel<1,2>"),
-                               "kernel": "store_kernel<1,2>", "ms_per_launch": store_ms,
+                               "frac": store_gbs / pk["hbm_gbs"], "traffic": traffic("store_kernel<1>"),
+                               "kernel": "store_kernel<1>", "ms_per_launch": store_ms,
                                "peak_source": pk["source"]},
             "gpu_launches": 4 * args.steps,
             "clocks": clk}
@@ -763,9 +789,9 @@ def run_batched(args):
     r, red = B.results()
     counts = [x.count for x in red]
     sols = sum(counts)
-    ops = batched_ops(B.Ws, counts)
+    ops = batched_ops(B.Ws, counts, walk_ops)
     ipk, ipk_basis = int_peak()
-    alu_ops = batched_ops(B.Ws, counts, alu_pipe_ops_per_solution)
+    alu_ops = batched_ops(B.Ws, counts, walk_alu_ops)
     apk, apk_basis = alu_pipe_peak()
     # the two-call form of the same work
     for _ in range(2):
@@ -812,11 +838,11 @@ def run_batched(args):
             "launch": "one persistent kernel (+3 memsets) replayed from a CUDA graph",
             "roofline": {"bound": "alu", "achieved": ops / (ms / 1e3) / 1e12, "peak": ipk,
                          "unit": "Tops/s", "frac": ops / (ms / 1e3) / 1e12 / ipk,
-                         "ops_per_batch": ops, "ops_per_solution": "22W - 4 (18 at W = 1)",
+                         "ops_per_batch": ops, "ops_per_solution": "20W - 2 (18 at W = 1)",
                          "kernel": "batch_kernel", "peak_basis": ipk_basis},
             "roofline_alu_pipe": {"bound": "alu_pipe", "achieved": alu_ops / (ms / 1e3) / 1e12, "peak": apk,
                                   "unit": "Tops/s", "frac": alu_ops / (ms / 1e3) / 1e12 / apk,
-                                  "ops_per_batch": alu_ops, "ops_per_solution": "16W - 4 (12 at W = 1)",
+                                  "ops_per_batch": alu_ops, "ops_per_solution": "14W - 2 (12 at W = 1)",
                                   "kernel": "batch_kernel", "peak_basis": apk_basis + " (the pipe that binds)"},
             "split_calls_ms_per_batch": split_ms,
             "store": {"what": "hlf_enumerate_batched storing min(2^r, 2^14) solutions of every grid",
@@ -936,7 +962,8 @@ def run_sharded(args, world, rank, local):
     k_ms = max_over_ranks(statistics.mean(e[0].elapsed_time(e[1]) for e in evs), world)
     mine = shard.shard_range(0, total, rank, world)[1]
     ipk, ipk_basis = int_peak(dev)
-    achieved = mine * ops_per_solution(W) / (k_ms / 1e3) / 1e12
+    red_kernel, red_ops, _ = headline_reduce(W, mine)
+    achieved = mine * red_ops / (k_ms / 1e3) / 1e12
     if rank != 0:
         return
     value = args.steps * total / dt
@@ -947,9 +974,9 @@ def run_sharded(args, world, rank, local):
             "warmup": max(3, args.warmup), "ms_per_step": 1e3 * dt / args.steps, "higher_is_better": True,
             "scaling": "strong", "vs_baseline": None, "dtype": "u64", "data": "synthetic", "config": cfg,
             "roofline": {"bound": "alu", "achieved": achieved, "peak": ipk, "unit": "Tops/s",
-                         "frac": achieved / ipk, "traffic": None, "kernel": "reduce_kernel<1,6,1024>",
+                         "frac": achieved / ipk, "traffic": None, "kernel": red_kernel,
                          "ms_per_launch": k_ms, "peak_basis": ipk_basis,
-                         "ops_per_solution": ops_per_solution(W)},
+                         "ops_per_solution": red_ops},
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": A_host.numel() * 8,
                     "d2h_bytes_per_step": red_host.numel() * 8,
                     "note": "the step itself runs through host buffers: A in, the partial out, the exchange"},

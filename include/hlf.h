@@ -188,7 +188,7 @@ hlf_status hlf_enumerate_store(hlf_handle* h, uint64_t offset, uint64_t count, u
  * Work on `stream` first waits for the factor kernel's stream.
  * out_dev: device, caller-owned, cap * W uint64, 8-byte aligned. Requires
  * cap <= HLF_STORE_UPTO_MAX (else HLF_ERR_ARG). Each solution is computed
- * from its index with up to r row XORs, so large windows belong to
+ * from its index with a lookup per four bits, so large windows belong to
  * hlf_enumerate_store.
  */
 #define HLF_STORE_UPTO_MAX (1ull << 24)

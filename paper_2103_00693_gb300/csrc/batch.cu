@@ -19,8 +19,8 @@
 //
 // Launch shape. One kernel per CTA size T = 64, 128 or 256 threads (2, 4 or
 // 8 warps per work item, chosen by the autotuner): every item, factorisation
-// or chunk, is worked on by one CTA, and a CTA of T threads holds 256 / T
-// rows of a matrix per thread. Smaller CTAs factor more instances at once
+// or chunk, is worked on by one CTA; of its warps one searches pivots and the others
+// hold the rows of a matrix (two warps: eight rows a thread). Smaller CTAs factor more instances at once
 // (more CTAs per SM); larger ones walk a chunk with more threads.
 //
 // Every wait is bounded: after spin_limit polls the chunk is skipped and

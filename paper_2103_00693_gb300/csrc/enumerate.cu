@@ -33,8 +33,6 @@
 namespace hlf {
 namespace {
 
-
-
 // The reduce of n_chunks windows of `chunk` indices, window c starting at
 // offset + c * chunk (hlf_enumerate_reduce is one window). A window is cut into
 // `parts` CTAs of blockDim.x threads, each thread walking `per` consecutive

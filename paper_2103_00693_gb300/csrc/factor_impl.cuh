@@ -125,8 +125,8 @@ __device__ __forceinline__ uint64_t* factor_rows(unsigned char* smem)
 // by their number mod 4. The searching warp is a serial chain of instructions, so
 // it has a scheduler to itself: it is warp 3, the row warps are those whose number
 // is not 3 mod 4, and the others stand idle until the elimination is done. Next to
-// row warps on its scheduler the search of a panel took up to twice as long (n =
-// 1024). A CTA of fewer than four warps has its last warp search.
+// row warps on its scheduler the searches took a fifth longer (n = 1024: 181k cycles
+// in all against 147k). A CTA of fewer than four warps has its last warp search.
 __host__ __device__ constexpr int search_warp(int nwarps) { return nwarps >= 4 ? 3 : nwarps - 1; }
 __host__ __device__ constexpr int row_warps(int nwarps) { return nwarps >= 4 ? nwarps - nwarps / 4 : nwarps - 1; }
 // The threads of a CTA with at least `want` row threads.
@@ -225,12 +225,15 @@ __device__ void eliminate_warp(const uint64_t* __restrict__ A, int n, unsigned c
 // with the next column's first); of several equal in both any may be, and the
 // one whose row ends up in prow is. The pivot's slice and set move to the pivot
 // slot of lane b, where later pivots clear their columns; the set ends as H_b.
-// A column is about 45 cycles; with a find-first and shuffles instead of the
-// maxima, and a branch where there is no pivot, it was 200.
+// A column takes 60, 77 or 109 cycles with 1, 2 or 4 slices a lane; with a ballot, a
+// find-first and shuffles instead of the maxima it took 200. Two halves of 16 columns
+// with slice and record in one word, one maximum a column, were slower (68, 91, 138):
+// the maximum's result is held in a uniform register, and what is formed from it
+// before it meets the slices lengthens the chain; joining the halves costs the rest.
 //
 // The loop runs eight columns per turn with the slices shifted up by eight after
 // each (what they shift out is zero in every candidate), so that its code stays
-// in the instruction cache: unrolled over 32 columns it ran half as fast.
+// in the instruction cache (unrolled over 32, a first run took 1.4 times a warm one).
 template <int NS, typename Smem>
 __device__ __forceinline__ uint32_t panel_search(Smem& sm, int16_t* prow, int nl, int p, int lane)
 {

@@ -1,9 +1,9 @@
-// Measurement helper behind the histogram's roofline: the rate at which this
-// GPU retires 32-bit shared-memory atomic adds. The paper has no counterpart;
+// Measurement helper: the rate at which this GPU retires 32-bit shared-memory
+// atomic adds, what counting solutions one by one could reach. The paper has no
+// counterpart;
 // the kernel does none of the method's arithmetic. Every thread of one full
 // wave of CTAs adds 1 to `iters` counters; the 32 lanes of a warp always hit
-// 32 distinct banks (the pattern of the histogram's interleaved walk when its
-// lanes land in distinct bins), and the counter addresses are compile-time
+// 32 distinct banks, and the counter addresses are compile-time
 // offsets from one register, so each atomic is one instruction with no
 // address arithmetic around it.
 
