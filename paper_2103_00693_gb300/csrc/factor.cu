@@ -135,8 +135,9 @@ __global__ void __launch_bounds__(factor_threads<W>(64 * W), 1) factor_elim_kern
 // q(x_f) = sum over i in supp(x_f) of popcount(A_i & x_f) mod 4, and
 // z^a_f = q(x_f) / 2 (z^a vanishes on the pivots). Each thread takes every
 // 256th k and every 256th row, so a free column costs a few rounds of
-// memory latency, not one per row. The paper-order table is built by warp 1
-// of CTA 0, as in factor_block. The last CTA to finish folds the checking
+// memory latency, not one per row. Word v of the paper-order table is built by warp
+// 1 of CTA v (all of it in one warp, rows in a chain, outlasted the free columns:
+// 18 us against 11 at n = 1024, cold). The last CTA to finish folds the checking
 // CTAs' verdicts and the q parity into the status word.
 template <int W>
 __global__ void __launch_bounds__(256) factor_kvec_kernel(const uint64_t* __restrict__ A, int n, FactorOut o,
@@ -165,21 +166,25 @@ __global__ void __launch_bounds__(256) factor_kvec_kernel(const uint64_t* __rest
         s_mask[lane] = fm;
         s_before[lane] = incl - cnt;
     }
-    if (blockIdx.x == 0 && warp == 1 && o.ptable && lane < W) {
-        // the paper's order: row l = XOR of A's columns (= rows) at p_{r-1}, .., p_{r-1-l}
+    if (blockIdx.x < W && warp == 1 && o.ptable) {
+        // the paper's order, word v of it by CTA v: row l = XOR of A's columns (= rows) at
+        // p_{r-1}, .., p_{r-1-l}; lane l has rows l and l + 32, two scans
+        const int v = blockIdx.x;
         const int nb = r < HLF_MAX_VARYING ? r : HLF_MAX_VARYING;
-        uint64_t acc = 0;
-        for (int l0 = 0; l0 < nb; l0 += 8) {  // eight independent loads in flight
-            uint64_t a[8];
+        uint64_t t0 = lane < nb ? A[(size_t)__ldcg(o.piv + r - 1 - lane) * W + v] : 0ull;
+        uint64_t t1 = lane + 32 < nb ? A[(size_t)__ldcg(o.piv + r - 33 - lane) * W + v] : 0ull;
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                a[u] = l0 + u < nb ? A[(size_t)__ldcg(o.piv + r - 1 - l0 - u) * W + lane] : 0ull;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                acc ^= a[u];
-                if (l0 + u < nb) o.ptable[(l0 + u) * W + lane] = acc;
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint64_t u0 = __shfl_up_sync(0xffffffffu, t0, d);
+            const uint64_t u1 = __shfl_up_sync(0xffffffffu, t1, d);
+            if (lane >= d) {
+                t0 ^= u0;
+                t1 ^= u1;
             }
         }
+        t1 ^= __shfl_sync(0xffffffffu, t0, 31);
+        if (lane < nb) o.ptable[lane * W + v] = t0;
+        if (lane + 32 < nb) o.ptable[(lane + 32) * W + v] = t1;
     }
     __syncthreads();
 
