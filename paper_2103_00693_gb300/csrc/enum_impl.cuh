@@ -438,35 +438,42 @@ struct Groups {
 };
 
 // Groups [h_first, h_end) of the window [offset, offset + count), group h being the
-// indices G h + odd .. G h + odd + G - 1, and the indices before and after them.
+// indices G h + phase .. G h + phase + G - 1, and the indices before and after them.
 struct GroupPlan {
     uint64_t n_head;      // [offset, offset + n_head)
     uint64_t tail_first;  // [tail_first, tail_first + n_tail)
     uint64_t n_tail;
     uint64_t h_first, h_end;
-    uint32_t odd;
+    uint32_t phase;
 };
 
-// odd (W = 1): pairs start at odd indices, so that they lie on 16 bytes where the
-// window's offset is odd; lane l then stores z(G h + 2 l + 1) and the next lane's
-// first solution (1.07 GB at an odd offset: 171 us, 198 with 8-byte stores). The window may end at 2^64 exactly, which wraps to 0.
-inline GroupPlan plan_groups(uint64_t offset, uint64_t count, uint64_t G, uint32_t odd)
+// phase < 4 (W = 1): where the groups start, such that they lie on 32 bytes whatever
+// the window's offset: lane l then stores z(G h + 2 l + phase) and the one after it,
+// which are its own or its neighbours'. 2^27 solutions take 171 us at every offset; with
+// groups at multiples of G they took 190 at offsets 2 mod 4 (a sector in two pieces
+// at each end of a step) and 234-246 at odd ones (8-byte stores). The window may end at
+// 2^64 exactly, which wraps to 0.
+inline uint32_t store_phase(const uint64_t* out, uint64_t offset)
+{
+    return (uint32_t)(offset - (reinterpret_cast<uintptr_t>(out) >> 3)) & 3;
+}
+inline GroupPlan plan_groups(uint64_t offset, uint64_t count, uint64_t G, uint32_t phase)
 {
     GroupPlan pl{};
-    pl.odd = odd;
+    pl.phase = phase;
     const uint64_t end = offset + count;  // 0 for 2^64
     const bool wraps = count != 0 && end == 0;
     // first group at or after offset, and one past the last that ends by `end`
-    const uint64_t h_first = offset <= odd ? 0 : (offset - odd - 1) / G + 1;
-    const uint64_t h_end = wraps && !odd ? (0ull - G) / G + 1 : (end < odd && !wraps ? 0 : (end - odd) / G);
+    const uint64_t h_first = offset <= phase ? 0 : (offset - phase - 1) / G + 1;
+    const uint64_t h_end = wraps && !phase ? (0ull - G) / G + 1 : (end < phase && !wraps ? 0 : (end - phase) / G);
     if (h_end <= h_first) {
         pl.n_head = count;
         return pl;
     }
     pl.h_first = h_first;
     pl.h_end = h_end;
-    pl.n_head = h_first * G + odd - offset;
-    pl.tail_first = h_end * G + odd;  // wraps to 0 only when the tail is empty
+    pl.n_head = h_first * G + phase - offset;
+    pl.tail_first = h_end * G + phase;  // wraps to 0 only when the tail is empty
     pl.n_tail = count - pl.n_head - (h_end - h_first) * G;
     return pl;
 }
@@ -549,10 +556,10 @@ __device__ __forceinline__ void store_ragged(Row row, const GroupPlan& g, uint64
 
 // Groups [h, h1) of a window, h < h1, by one warp from the lanes' seeds: `dst` is the
 // output less offset * W words, `step(j)` points to C_j, `b0` is B_0's word (W = 1),
-// `stage` holds stage_words<W>() words of the warp (W > 1). W = 1 needs dst + odd on
-// 16 bytes or `pairs` false, W > 1 dst on 16 bytes.
+// `stage` holds stage_words<W>() words of the warp (W > 1, where phase is 0 and dst lies
+// on 16 bytes).
 template <int W, typename Step, typename Check>
-__device__ __forceinline__ void store_groups(uint64_t (&z)[W], uint64_t h, uint64_t h1, uint32_t odd, uint64_t b0,
+__device__ __forceinline__ void store_groups(uint64_t (&z)[W], uint64_t h, uint64_t h1, uint32_t phase, uint64_t b0,
                                              uint64_t* dst, uint64_t* stage, int lane, Step step, Check ok)
 {
     constexpr uint64_t G = Groups<W>::kSize;
@@ -560,13 +567,22 @@ __device__ __forceinline__ void store_groups(uint64_t (&z)[W], uint64_t h, uint6
         for (;;) {
             const uint64_t z1 = z[0] ^ b0;  // g(2t + 1) = g(2t) ^ 1
             const uint64_t zn = z[0] ^ step(ctz64(h + 1))[0];
-            const uint64_t i = h * G + 2 * lane + odd;
-            if (odd) {  // warp-uniform
+            const uint64_t i = h * G + 2 * lane + phase;
+            uint64_t a = z[0], b = z1;
+            if (phase) {  // warp-uniform; the last lanes' neighbours are in the next group
                 const uint64_t next = __shfl_sync(0xffffffffu, lane == 0 ? zn : z[0], (lane + 1) & 31);
-                if (ok(i, 2)) st_cs_v2(dst + i, z1, next);
-            } else {
-                if (ok(i, 2)) st_cs_v2(dst + i, z[0], z1);
+                if (phase == 1) {
+                    a = z1;
+                    b = next;
+                } else if (phase == 2) {
+                    a = next;
+                    b = next ^ b0;
+                } else {
+                    a = next ^ b0;
+                    b = __shfl_sync(0xffffffffu, lane < 2 ? zn : z[0], (lane + 2) & 31);
+                }
             }
+            if (ok(i, 2)) st_cs_v2(dst + i, a, b);
             if (++h == h1) break;
             z[0] = zn;
         }

@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kThreads) store_kernel(const uint64_t* __restr
     const uint64_t h1 = min(h0 + pl.per_warp, pl.g.h_end);
     uint64_t z[W];
     seed_group<W>(row, h0, lane, z);
-    store_groups<W>(z, h0, h1, pl.g.odd, t.B[0][0], out - pl.offset * W,
+    store_groups<W>(z, h0, h1, pl.g.phase, t.B[0][0], out - pl.offset * W,
                     s_stage + (threadIdx.x >> 5) * stage_words<W>(), lane, [&](int j) { return s_C[j]; }, ok);
 }
 
@@ -493,9 +493,7 @@ hlf_status launch_store_w(const uint64_t* table, uint64_t offset, uint64_t count
     StorePlan pl{};
     pl.offset = offset;
     pl.count = count;
-    // W = 1: pairs on 16 bytes, whichever the parity of the window's first word
-    const uint32_t odd = W == 1 ? ((reinterpret_cast<uintptr_t>(out) >> 3) ^ offset) & 1 : 0;
-    pl.g = plan_groups(offset, count, Groups<W>::kSize, odd);
+    pl.g = plan_groups(offset, count, Groups<W>::kSize, W == 1 ? store_phase(out, offset) : 0);
     const uint64_t groups = pl.g.h_end - pl.g.h_first;
     constexpr size_t smem_warp = W == 1 ? 0 : stage_words<W>() * sizeof(uint64_t);
     constexpr size_t smem_max = smem_warp * (kThreads / 32);

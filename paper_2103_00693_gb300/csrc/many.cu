@@ -60,7 +60,7 @@ __device__ void many_tasks(const WinDesc& d, uint64_t u, uint64_t u1, int lane, 
     __syncwarp();
     uint64_t rare[W];  // a step row that is not staged
     store_groups<W>(
-        z, h0, h1, d.g.odd, __ldg(tab), d.out - d.offset * W, stage, lane,
+        z, h0, h1, d.g.phase, __ldg(tab), d.out - d.offset * W, stage, lane,
         [&](int j) -> const uint64_t* {
             if (j < kTaskRows) return C + j * W;
 #pragma unroll
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kThreads, 2) many_kernel(const WinDesc* __rest
 void plan_window(WinDesc& d, uint32_t W)
 {
     const uint64_t G = W == 1 ? Groups<1>::kSize : Groups<2>::kSize;
-    d.g = plan_groups(d.offset, d.count, G, W == 1 ? d.offset & 1 : 0);
+    d.g = plan_groups(d.offset, d.count, G, W == 1 ? store_phase(d.out, d.offset) : 0);
     d.W = W;
     const uint64_t tg = task_groups(W);
     d.ntasks = (uint32_t)(ragged_shares(d.g) + (d.g.h_end - d.g.h_first + tg - 1) / tg);
