@@ -75,9 +75,9 @@ KERNEL_SOURCES = {
     "dense1_kernel<16,1,1>": ["dense.cu", "enum_impl.cuh", "hlf_internal.cuh"],
 }
 TRAFFIC = {  # kernel -> per-launch DRAM bytes (read + write) and the source digest at capture
-    "reduce_region_kernel": {"bytes": 541440 + 1536, "sources": "0b975b98a6be7595"},
-    "store_kernel<1>": {"bytes": 244992 + 8525198848, "sources": "0b975b98a6be7595"},
-    "dense1_kernel<16,1,1>": {"bytes": 467200 + 4767411200, "sources": "2a92c04830996b04"},
+    "reduce_region_kernel": {"bytes": 802816, "sources": "3dea016f284bb1a9"},
+    "store_kernel<1>": {"bytes": 113408 + 8525068032, "sources": "3dea016f284bb1a9"},
+    "dense1_kernel<16,1,1>": {"bytes": 54016 + 4766962176, "sources": "1ed5ba2bef1e06b7"},
 }
 
 
