@@ -20,8 +20,8 @@
 // barrier per column; up to n = 256 every row took the pivot row's words each
 // column) and now:
 //   grid, p = 1/2        n = 100: 21.2 -> 14.4 us   256: 50.7 -> 28.7
-//                        484: 81.8 -> 50.4          1024: 202 -> 105
-//   random symmetric     n = 256: 47.4 -> 24.7      1024: 309 -> 220
+//                        484: 81.8 -> 47.2          1024: 202 -> 100
+//   random symmetric     n = 256: 47.4 -> 24.7      1024: 309 -> 214
 // Per panel of 32 columns at n = 1024 (cycles): the search 4100 on a grid and 5200
 // on a dense matrix (with a warp to itself and nothing else on the SM 1900 to 3500,
 // by how many slices are live), the list and the first word's tables and updates
@@ -89,6 +89,7 @@ __device__ void eliminate_only(const uint64_t* __restrict__ A, int n, const Fact
     FactorSmem<W, HLF_MAX_N>& sm = *reinterpret_cast<FactorSmem<W, HLF_MAX_N>*>(smem);
     const int tid = threadIdx.x;
     eliminate_panels<W, R, HLF_MAX_N>(A, n, smem, nullptr, [](int, int) {});
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = order_pivots(sm, n);
     const int nb = r < HLF_MAX_VARYING ? r : HLF_MAX_VARYING;
     write_basis(sm, factor_rows<W, HLF_MAX_N>(smem), n, r, o, kTableTotalRows);
@@ -151,6 +152,7 @@ __global__ void __launch_bounds__(256) factor_kvec_kernel(const uint64_t* __rest
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int warp = tid >> 5;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int r = __ldcg(o.work + kWorkR);
     if (warp == 0) {
         const int c0 = lane * 32;
@@ -281,8 +283,18 @@ hlf_status launch_factor_large(const uint64_t* A, int n, const FactorOut& o, cud
     }
     factor_elim_kernel<W><<<1 + kChkCtas, factor_threads<W>(n), smem, s>>>(A, n, o);
     if (cudaGetLastError() != cudaSuccess) return HLF_ERR_CUDA;
-    factor_kvec_kernel<W><<<kKvecCtas, 256, 0, s>>>(A, n, o, kChkCtas);
-    return cudaGetLastError() == cudaSuccess ? HLF_OK : HLF_ERR_CUDA;
+    // launched when the elimination has only its results to write: grid 32 x 32 102.7 ->
+    // 100.4 us, random symmetric n = 700 107.0 -> 105.2, n = 1024 216.4 -> 214.4
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = kKvecCtas;
+    cfg.blockDim = 256;
+    cfg.stream = s;
+    cudaLaunchAttribute beside{};
+    beside.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    beside.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &beside;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, factor_kvec_kernel<W>, A, n, o, (int)kChkCtas) == cudaSuccess ? HLF_OK : HLF_ERR_CUDA;
 }
 
 }  // namespace
