@@ -20,13 +20,14 @@
 // barrier per column; up to n = 256 every row took the pivot row's words each
 // column) and now:
 //   grid, p = 1/2        n = 100: 21.2 -> 14.4 us   256: 50.7 -> 28.7
-//                        484: 81.8 -> 47.2          1024: 202 -> 100
-//   random symmetric     n = 256: 47.4 -> 24.7      1024: 309 -> 214
+//                        484: 81.8 -> 47.2          1024: 202 -> 99
+//   random symmetric     n = 256: 47.4 -> 24.7      1024: 309 -> 200
 // Per panel of 32 columns at n = 1024 (cycles): the search 4100 on a grid and 5200
 // on a dense matrix (with a warp to itself and nothing else on the SM 1900 to 3500,
 // by how many slices are live), the list and the first word's tables and updates
 // 1000; the other words' tables and updates, 3000 on a grid, are hidden behind the
-// next search, and 8800 on a dense matrix, where shared-memory reads bound them.
+// next search; on a dense matrix their shared-memory reads (5900 cycles of bandwidth a
+// panel at first) are what it waits for.
 //
 // Measured on the way: the search by ballot, find-first and shuffles instead of
 // maxima 200 cycles a column against 60 to 110; the words dealt to their rows' owners

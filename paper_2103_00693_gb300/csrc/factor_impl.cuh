@@ -302,6 +302,11 @@ __device__ __forceinline__ uint32_t panel_search(Smem& sm, int16_t* prow, int nl
     return cols;
 }
 
+template <int N>
+struct Words {
+    static constexpr int value = N;
+};
+
 // W > 1: the elimination by panels of 32 columns, in a CTA of row threads (R rows
 // each: t, t + row threads, ...) and one more warp that searches.
 //
@@ -405,7 +410,8 @@ __device__ void eliminate_panels(const uint64_t* __restrict__ A, int n, unsigned
     };
     // Words w_from.. but w_done still lack the last panel's update. The rows that
     // need it (on a grid, those near the panel) are listed and their words dealt to
-    // all row warps: 32 rows and kTaskWords words a task.
+    // all row warps: 32 rows and kTaskWords words a task, whose loads are all in flight at
+    // once (random symmetric n = 1024: 200 us; word by word 214, n = 700: 100 and 105).
     constexpr int kTaskWords = 4;
     int w_from = W, w_done = 0;
     auto finish = [&]() {
@@ -427,7 +433,7 @@ __device__ void eliminate_panels(const uint64_t* __restrict__ A, int n, unsigned
         bar_rows();
         const int na = sm.nactive;
         const int chunks = (na + 31) >> 5;
-        int ch = tid >> 5, v0 = w_from;
+        int ch = tid >> 5, v0 = w_from + 1;  // w_from itself is done, or takes w_from + 1's place, which is
         for (;;) {
             while (ch >= chunks && v0 < W) {
                 ch -= chunks;
@@ -441,13 +447,23 @@ __device__ void eliminate_panels(const uint64_t* __restrict__ A, int n, unsigned
 #pragma unroll
                 for (int t = 0; t < 8; ++t) tb[t] = T2 + (t * W + v0) * 16 + ((rc.y >> (4 * t)) & 15u);
                 uint64_t* x = rows + v0 * S + rc.x;
-#pragma unroll 2
-                for (int i = 0; i < kTaskWords; ++i) {
-                    if (v0 + i >= W) break;
-                    if (v0 + i == w_done) continue;
-                    x[i * S] ^= ((tb[0][16 * i] ^ tb[1][16 * i]) ^ (tb[2][16 * i] ^ tb[3][16 * i])) ^
-                                ((tb[4][16 * i] ^ tb[5][16 * i]) ^ (tb[6][16 * i] ^ tb[7][16 * i]));
-                }
+                const int first = v0 == w_done ? -1 : 0;
+                auto task = [&](auto words) {  // all the loads in flight
+                    constexpr int N = decltype(words)::value;
+                    uint64_t acc[N];
+#pragma unroll
+                    for (int i = 0; i < N; ++i) acc[i] = x[(i ? i : first) * S];
+#pragma unroll
+                    for (int t = 0; t < 8; ++t)
+#pragma unroll
+                        for (int i = 0; i < N; ++i) acc[i] ^= tb[t][16 * (i ? i : first)];
+#pragma unroll
+                    for (int i = 0; i < N; ++i) x[(i ? i : first) * S] = acc[i];
+                };
+                if (v0 + kTaskWords <= W) task(Words<kTaskWords>{});
+                else if (v0 + 3 == W) task(Words<3>{});
+                else if (v0 + 2 == W) task(Words<2>{});
+                else task(Words<1>{});
             }
             ch += rt >> 5;
         }
