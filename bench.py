@@ -75,8 +75,8 @@ KERNEL_SOURCES = {
     "dense1_kernel<16,1,1>": ["dense.cu", "enum_impl.cuh", "hlf_internal.cuh"],
 }
 TRAFFIC = {  # kernel -> per-launch DRAM bytes (read + write) and the source digest at capture
-    "reduce_region_kernel": {"bytes": 802816, "sources": "3dea016f284bb1a9"},
-    "store_kernel<1>": {"bytes": 113408 + 8525068032, "sources": "3dea016f284bb1a9"},
+    "reduce_region_kernel": {"bytes": 1044736, "sources": "aa64cb219d91c923"},
+    "store_kernel<1>": {"bytes": 270080 + 8524897536, "sources": "aa64cb219d91c923"},
     "dense1_kernel<16,1,1>": {"bytes": 54016 + 4766962176, "sources": "1ed5ba2bef1e06b7"},
 }
 
