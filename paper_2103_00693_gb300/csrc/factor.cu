@@ -90,8 +90,10 @@ __device__ void eliminate_only(const uint64_t* __restrict__ A, int n, const Fact
     FactorSmem<W, HLF_MAX_N>& sm = *reinterpret_cast<FactorSmem<W, HLF_MAX_N>*>(smem);
     const int tid = threadIdx.x;
     eliminate_panels<W, R, HLF_MAX_N>(A, n, smem, nullptr, [](int, int) {});
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = order_pivots(sm, n);
+    // Behind order_pivots' barriers: a CTA releases its dependents when the first of its
+    // threads does, and the idle warps leave the elimination at its start.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int nb = r < HLF_MAX_VARYING ? r : HLF_MAX_VARYING;
     write_basis(sm, factor_rows<W, HLF_MAX_N>(smem), n, r, o, kTableTotalRows);
     if (o.ptable)
@@ -284,8 +286,12 @@ hlf_status launch_factor_large(const uint64_t* A, int n, const FactorOut& o, cud
     }
     factor_elim_kernel<W><<<1 + kChkCtas, factor_threads<W>(n), smem, s>>>(A, n, o);
     if (cudaGetLastError() != cudaSuccess) return HLF_ERR_CUDA;
-    // launched when the elimination has only its results to write: grid 32 x 32 102.7 ->
-    // 100.4 us, random symmetric n = 700 107.0 -> 105.2, n = 1024 216.4 -> 214.4
+    // Launched when the elimination has only its results to write: grid 32 x 32 102.5 us
+    // (104.5 launched when it has ended), random symmetric n = 700 89.9 (92.4), n = 1024
+    // 200.8 (202.9). Not sooner: its CTAs wait on every SM, and other streams' kernels of
+    // large CTAs find no room beside them. Released at the elimination's start, 8
+    // factorisations of n = 1024 on 8 streams took 391 us (now 221), and a reduce of 40 us
+    // on another stream 208 (now 44).
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = kKvecCtas;
     cfg.blockDim = 256;
