@@ -29,6 +29,7 @@
 //   sample_kernel        z(i) at arbitrary indices, straight from the formula.
 
 #include "enum_impl.cuh"
+#include "reduce_cut.h"
 
 namespace hlf {
 namespace {
@@ -37,7 +38,8 @@ namespace {
 // offset + c * chunk (hlf_enumerate_reduce is one window). A window is cut into
 // `parts` CTAs of blockDim.x threads, each thread walking `per` consecutive
 // indices that start at a multiple of 2^U, so that only the window's two ends
-// have partial Gray blocks. Items (window, part) are taken grid-stride. With
+// have partial Gray blocks; a window of few blocks (align = 0) is dealt from its own
+// start. Items (window, part) are taken grid-stride. With
 // one part per window the CTA writes the result unless asked to add; otherwise it
 // adds to it, once the kernel that clears the results (clear_results_kernel, which this
 // one may start beside) has ended.
@@ -360,83 +362,13 @@ int blocks_per_sm(K kernel, size_t smem)
     return fit;
 }
 
-// How a reduce of n_chunks windows of `chunk` indices is cut: CTAs of
-// `threads`, `parts` of them per window, `per` indices per thread.
-struct ReduceShape {
-    unsigned threads, blocks;
-    uint32_t parts;
-    uint64_t per, runs;
-    uint64_t align;  // runs start at multiples of align + 1
-};
-
-// The threads a window can use are one per Gray block of 2^U indices; a seed
-// costs a few tens of solutions (kSeedCost), so short runs are worth it
-// whenever they fill idle SMs. One window: one CTA if that holds them all (the
-// result then needs no clearing), else all of them, up to one wave, in CTAs no
-// larger than spreading them over every SM takes. Several windows: the CTA size and
-// the cut whose waves cost least.
-// With runs of at least 2048 indices and one CTA per window instead, 2^20
-// four-word solutions took 694 us on one SM (now 10.8, two launches and the
-// host's call among it), and 64 windows of 2^24 at W = 1 took 2.16 ms on 64
-// CTAs of 256 threads (now 0.79).
-template <int W, int U, int T>
-ReduceShape reduce_shape(uint64_t chunk, uint64_t n_chunks)
-{
-    constexpr uint64_t kSeedCost = 48;
-    const uint64_t sms = (uint64_t)sm_count();
-    const uint64_t runs = ((chunk - 1) >> U) + 2;  // Gray blocks the window touches, at most
-    const uint64_t room = (uint64_t)min_ctas_for(W) * T;  // threads an SM holds
-    ReduceShape sh{};
-    uint64_t want;  // threads for the window
-    if (n_chunks == 1) {
-        want = runs < sms * room ? runs : sms * room;
-        uint64_t bd = want <= T ? want : (want + sms - 1) / sms;
-        bd = (bd + 31) / 32 * 32;
-        bd = bd > T ? T : (want > T && bd < 128 ? 128 : bd);
-        sh.threads = (unsigned)bd;
-        sh.parts = (uint32_t)((want + bd - 1) / bd);
-    } else {
-        // CTAs of T threads down to 64, 1 to 64 of them a window: the fewest steps of
-        // the busiest SM. Smaller CTAs only where that saves 1/16: each builds its own
-        // tables (64 windows of 2^24 in CTAs of 64 threads 813 us, of 1024 792, though
-        // the former fill the wave 3% better; 64 of 1239596 78 us against 82).
-        uint64_t best = ~0ull;
-        for (uint64_t bd = T; bd >= 64; bd /= 2) {
-            const uint64_t slots = sms * (room / bd);
-            const uint64_t least = best - best / 16;
-            for (uint64_t k = 1; k <= 64 && (k == 1 || (k - 1) * bd < runs); ++k) {
-                const uint64_t waves = (n_chunks * k + slots - 1) / slots;
-                const uint64_t cost = waves * (kSeedCost + (((chunk - 1) / (k * bd)) | ((1ull << U) - 1)) + 1);
-                if (cost < best && (bd == T || cost < least)) {
-                    best = cost;
-                    sh.parts = (uint32_t)k;
-                    sh.threads = (unsigned)bd;
-                }
-                if (n_chunks > (~0ull >> 8)) break;  // a window each is enough
-            }
-        }
-    }
-    want = (uint64_t)sh.parts * sh.threads;
-    // chunk + 2^U - 1 indices at most, counted from the window's first block;
-    // past 2^63 that count could wrap, so such windows start their runs at the
-    // window's own start
-    sh.align = chunk <= 1ull << 63 ? (1ull << U) - 1 : 0;
-    sh.per = chunk / want + (chunk % want + sh.align + want - 1) / want;
-    sh.per = (sh.per + (1ull << U) - 1) & ~((1ull << U) - 1);
-    sh.runs = sh.align ? want : (chunk - 1) / sh.per + 1;
-    const uint64_t items = n_chunks * sh.parts;
-    const uint64_t cap = sms * (room / sh.threads);
-    sh.blocks = (unsigned)(items < cap ? items : cap);
-    return sh;
-}
-
 // add: *out is a sum in progress (one window).
 template <int W, int U>
 hlf_status launch_reduce_u(const uint64_t* table, uint64_t offset, uint64_t chunk, uint64_t n_chunks,
                            hlf_reduce* out, cudaStream_t s, bool add = false)
 {
     constexpr int T = reduce_threads(W);
-    const ReduceShape sh = reduce_shape<W, U, T>(chunk, n_chunks);
+    const ReduceShape sh = reduce_shape(chunk, n_chunks, U, T, (uint64_t)sm_count(), (uint64_t)min_ctas_for(W) * T);
     const int ntab = seed_tables_for(offset + (chunk * n_chunks - 1));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = sh.blocks;

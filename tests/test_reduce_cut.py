@@ -1,0 +1,84 @@
+"""The cut of a reduce over CTAs and threads (csrc/reduce_cut.h), compiled for the host:
+every index of a window belongs to one thread, the grid is one wave at most, and a
+window of few Gray blocks is dealt to enough lanes."""
+
+import ctypes
+import random
+import subprocess
+
+import pytest
+
+from paper_2103_00693_gb300 import build as hbuild
+
+SHIM = """
+#include "reduce_cut.h"
+extern "C" void cut(uint64_t chunk, uint64_t n, int U, uint64_t T, uint64_t sms, uint64_t room, uint64_t* o)
+{
+    const hlf::ReduceShape s = hlf::reduce_shape(chunk, n, U, T, sms, room);
+    o[0] = s.threads; o[1] = s.blocks; o[2] = s.parts; o[3] = s.per; o[4] = s.runs; o[5] = s.align;
+}
+"""
+SMS = 152
+SHAPES = [(1, 3, 1024, 1024), (1, 6, 1024, 1024), (2, 4, 1024, 1024), (4, 3, 1024, 1024), (5, 2, 256, 512), (16, 2, 256, 512)]
+
+
+@pytest.fixture(scope="module")
+def cut(tmp_path_factory):
+    d = tmp_path_factory.mktemp("cut")
+    (d / "shim.cpp").write_text(SHIM)
+    subprocess.run(["g++", "-std=c++17", "-O2", "-shared", "-fPIC", "-I", hbuild.CSRC, str(d / "shim.cpp"), "-o",
+                    str(d / "cut.so")], check=True)
+    lib = ctypes.CDLL(str(d / "cut.so"))
+
+    def f(chunk, n, shape):
+        W, U, T, room = shape
+        o = (ctypes.c_uint64 * 6)()
+        u64 = ctypes.c_uint64
+        lib.cut(u64(chunk), u64(n), U, u64(T), u64(SMS), u64(room), o)
+        return dict(zip(("threads", "blocks", "parts", "per", "runs", "align"), o))
+
+    return f
+
+
+def _runs(s, first, chunk):
+    """The kernel's own arithmetic: (first index, length) of each thread's run."""
+    skip = first & s["align"]
+    for run in range(s["parts"] * s["threads"]):
+        a = run * s["per"]
+        lo = max(a, skip)
+        if run < s["runs"] and lo - skip < chunk:
+            yield first + lo - skip, min(s["per"] - (lo - a), chunk - (lo - skip))
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_every_index_once(cut, shape):
+    rng = random.Random(shape[0])
+    sizes = [1, 2, 3, 4, 7, 8, 15, 16, 31, 32, 33, 63, 64, 96, 97, 224, 225, 255, 256, 480, 481, 768, 769, 1023, 3840, 3841, 8191]
+    for chunk in sizes + [int(2 ** rng.uniform(0, 34)) for _ in range(12)]:
+        for n in (1, 7, 153, 100000):
+            s = cut(chunk, n, shape)
+            assert 32 <= s["threads"] <= shape[2] and s["threads"] % 32 == 0
+            assert 1 <= s["blocks"] <= min(n * s["parts"], SMS * (shape[3] // s["threads"]))
+            first = rng.randrange(1 << 40)
+            at = first
+            for i, length in _runs(s, first, chunk):
+                assert i == at and length >= 1, (chunk, n, s)
+                at += length
+            assert at == first + chunk, (chunk, n, s)
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_short_windows_fill_lanes(cut, shape):
+    """A thread of a short window walks no more than a warp's share of it; where all
+    windows run at once, no more than a CTA's."""
+    U = shape[1]
+    for chunk in (2, 10, 31, 32 * ((1 << U) - 1)):
+        assert cut(chunk, 100000, shape)["per"] <= (chunk + 31) // 32
+        assert cut(chunk, 7, shape)["per"] <= (chunk + 255) // 256
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_one_window_has_threads_for_its_tables(cut, shape):
+    for chunk in (1, 4, 20):
+        s = cut(chunk, 1, shape)
+        assert s["threads"] >= 256 and s["parts"] == 1
