@@ -368,7 +368,8 @@ hlf_status launch_reduce_u(const uint64_t* table, uint64_t offset, uint64_t chun
                            hlf_reduce* out, cudaStream_t s, bool add = false)
 {
     constexpr int T = reduce_threads(W);
-    const ReduceShape sh = reduce_shape(chunk, n_chunks, U, T, (uint64_t)sm_count(), (uint64_t)min_ctas_for(W) * T);
+    const ReduceShape sh = reduce_shape(chunk, n_chunks, U, T, (uint64_t)sm_count(), (uint64_t)min_ctas_for(W) * T,
+                                        sizeof(Table<W>) + sizeof(SeedTable<W>) + sizeof(uint64_t) * (T / 32) * (2 + W));
     const int ntab = seed_tables_for(offset + (chunk * n_chunks - 1));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = sh.blocks;

@@ -6,6 +6,9 @@
 
 namespace hlf {
 
+constexpr uint64_t kSmShared = 228 * 1024;  // shared memory of an SM
+constexpr uint64_t kCtaShared = 1024;       // of it kept per CTA by the system
+
 // CTAs of `threads`, `parts` of them per window, `per` indices per thread.
 struct ReduceShape {
     unsigned threads, blocks;
@@ -25,13 +28,20 @@ struct ReduceShape {
 // host's call among it), and 64 windows of 2^24 at W = 1 took 2.16 ms on 64
 // CTAs of 256 threads (now 0.79).
 //
-// U: log2 of the Gray block; T: the most threads of a CTA; room: threads an SM holds.
-inline ReduceShape reduce_shape(uint64_t chunk, uint64_t n_chunks, int U, uint64_t T, uint64_t sms, uint64_t room)
+// U: log2 of the Gray block; T: the most threads of a CTA; room: threads an SM's
+// registers hold; smem: a CTA's shared memory.
+inline ReduceShape reduce_shape(uint64_t chunk, uint64_t n_chunks, int U, uint64_t T, uint64_t sms, uint64_t room,
+                                uint64_t smem)
 {
     constexpr uint64_t kSeedCost = 48;
     // Threads that build a CTA's tables in good time: one solution of 16 words at an
     // index of 60 bits takes 8.3 us, with 32 of them 18.6.
     constexpr uint64_t kFew = 256;
+    // The seed tables bind small CTAs of wide rows: at W = 16 an SM holds five of them,
+    // not the eight of 64 threads that its registers would. Cut as if they fitted, 1000
+    // windows of 5000 took 153 us (now 125), 1216 of 5000 168 (128).
+    const uint64_t most = kSmShared / (smem + kCtaShared);
+    auto fit = [&](uint64_t threads) { return room / threads < most ? room / threads : most; };
     const uint64_t runs = ((chunk - 1) >> U) + 2;  // Gray blocks the window touches, at most
     ReduceShape sh{};
     uint64_t want;  // threads for the window
@@ -50,7 +60,7 @@ inline ReduceShape reduce_shape(uint64_t chunk, uint64_t n_chunks, int U, uint64
         // the former fill the wave 3% better; 64 of 1239596 78 us against 82).
         uint64_t best = ~0ull;
         for (uint64_t bd = T; bd >= 64; bd /= 2) {
-            const uint64_t slots = sms * (room / bd);
+            const uint64_t slots = sms * fit(bd);
             const uint64_t least = best - best / 16;
             for (uint64_t k = 1; k <= 64 && (k == 1 || (k - 1) * bd < runs); ++k) {
                 const uint64_t waves = (n_chunks * k + slots - 1) / slots;
@@ -64,7 +74,7 @@ inline ReduceShape reduce_shape(uint64_t chunk, uint64_t n_chunks, int U, uint64
             }
         }
     }
-    const uint64_t slots = sms * (room / sh.threads), items = n_chunks * sh.parts;
+    const uint64_t slots = sms * fit(sh.threads), items = n_chunks * sh.parts;
     sh.blocks = (unsigned)(items < slots ? items : slots);
     // A window with too few Gray blocks for the threads at hand, a CTA's if all windows
     // run at once, else those of a warp, is dealt to them by the index: idle lanes cost

@@ -12,14 +12,25 @@ from paper_2103_00693_gb300 import build as hbuild
 
 SHIM = """
 #include "reduce_cut.h"
-extern "C" void cut(uint64_t chunk, uint64_t n, int U, uint64_t T, uint64_t sms, uint64_t room, uint64_t* o)
+extern "C" void cut(uint64_t chunk, uint64_t n, int U, uint64_t T, uint64_t sms, uint64_t room, uint64_t smem, uint64_t* o)
 {
-    const hlf::ReduceShape s = hlf::reduce_shape(chunk, n, U, T, sms, room);
+    const hlf::ReduceShape s = hlf::reduce_shape(chunk, n, U, T, sms, room, smem);
     o[0] = s.threads; o[1] = s.blocks; o[2] = s.parts; o[3] = s.per; o[4] = s.runs; o[5] = s.align;
 }
 """
 SMS = 152
-SHAPES = [(1, 3, 1024, 1024), (1, 6, 1024, 1024), (2, 4, 1024, 1024), (4, 3, 1024, 1024), (5, 2, 256, 512), (16, 2, 256, 512)]
+SHAPES = [(1, 3, 1024, 1024), (1, 6, 1024, 1024), (2, 4, 1024, 1024), (4, 3, 1024, 1024), (5, 2, 256, 512), (11, 2, 256, 512), (16, 2, 256, 512)]
+
+
+def _smem(shape):
+    """A CTA's tables and partial results in bytes."""
+    W, _, T, _ = shape
+    return 66 * W * 8 + 16 * 16 * W * 8 + T // 32 * (2 + W) * 8
+
+
+def _fit(shape, threads):
+    """CTAs that an SM of 228 KB, 1 KB of it for each CTA, holds at once."""
+    return min(shape[3] // threads, 228 * 1024 // (_smem(shape) + 1024))
 
 
 @pytest.fixture(scope="module")
@@ -34,7 +45,7 @@ def cut(tmp_path_factory):
         W, U, T, room = shape
         o = (ctypes.c_uint64 * 6)()
         u64 = ctypes.c_uint64
-        lib.cut(u64(chunk), u64(n), U, u64(T), u64(SMS), u64(room), o)
+        lib.cut(u64(chunk), u64(n), U, u64(T), u64(SMS), u64(room), u64(_smem(shape)), o)
         return dict(zip(("threads", "blocks", "parts", "per", "runs", "align"), o))
 
     return f
@@ -58,7 +69,7 @@ def test_every_index_once(cut, shape):
         for n in (1, 7, 153, 100000):
             s = cut(chunk, n, shape)
             assert 32 <= s["threads"] <= shape[2] and s["threads"] % 32 == 0
-            assert 1 <= s["blocks"] <= min(n * s["parts"], SMS * (shape[3] // s["threads"]))
+            assert 1 <= s["blocks"] <= min(n * s["parts"], SMS * _fit(shape, s["threads"]))
             first = rng.randrange(1 << 40)
             at = first
             for i, length in _runs(s, first, chunk):
