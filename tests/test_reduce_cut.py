@@ -11,7 +11,26 @@ import pytest
 from paper_2103_00693_gb300 import build as hbuild
 
 SHIM = """
+#include <chrono>
 #include "reduce_cut.h"
+using Clock = std::chrono::steady_clock;
+extern "C" double divisions(uint64_t chunk, uint64_t n, int U, uint64_t T, uint64_t sms, uint64_t room, uint64_t smem)
+{
+    volatile uint64_t c = chunk, by = 3, sink = 0;
+    double best = 1e30;
+    for (int rep = 0; rep < 20; ++rep) {
+        uint64_t x = 0, y = ~0ull;
+        const auto t0 = Clock::now();
+        for (int i = 0; i < 500; ++i) x += hlf::reduce_shape(c, n, U, T, sms, room, smem).per;
+        const auto t1 = Clock::now();
+        for (int i = 0; i < 500 * 100; ++i) y = (y + ~0ull) / by;
+        const auto t2 = Clock::now();
+        sink = x + y;
+        const double r = 100.0 * (t1 - t0).count() / (t2 - t1).count();
+        if (r < best) best = r;
+    }
+    return best;
+}
 extern "C" void cut(uint64_t chunk, uint64_t n, int U, uint64_t T, uint64_t sms, uint64_t room, uint64_t smem, uint64_t* o)
 {
     const hlf::ReduceShape s = hlf::reduce_shape(chunk, n, U, T, sms, room, smem);
@@ -41,10 +60,14 @@ def cut(tmp_path_factory):
                     str(d / "cut.so")], check=True)
     lib = ctypes.CDLL(str(d / "cut.so"))
 
-    def f(chunk, n, shape):
+    lib.divisions.restype = ctypes.c_double
+
+    def f(chunk, n, shape, divisions=False):
         W, U, T, room = shape
         o = (ctypes.c_uint64 * 6)()
         u64 = ctypes.c_uint64
+        if divisions:
+            return lib.divisions(u64(chunk), u64(n), U, u64(T), u64(SMS), u64(room), u64(_smem(shape)))
         lib.cut(u64(chunk), u64(n), U, u64(T), u64(SMS), u64(room), u64(_smem(shape)), o)
         return dict(zip(("threads", "blocks", "parts", "per", "runs", "align"), o))
 
@@ -93,3 +116,36 @@ def test_one_window_has_threads_for_its_tables(cut, shape):
     for chunk in (1, 4, 20):
         s = cut(chunk, 1, shape)
         assert s["threads"] >= 256 and s["parts"] == 1
+
+
+def _every_cut(chunk, n, shape):
+    """(threads, parts) of the first cheapest cut, each tried by itself."""
+    W, U, T, _ = shape
+    runs, best, pick = ((chunk - 1) >> U) + 2, 1 << 64, None
+    bd = T
+    while bd >= 64:
+        slots, least, k = SMS * _fit(shape, bd), best - best // 16, 1
+        while k <= 64 and (k == 1 or (k - 1) * bd < runs):
+            cost = -(-n * k // slots) * (48 + ((chunk - 1) // (k * bd) | (1 << U) - 1) + 1)
+            if cost < best and (bd == T or cost < least):
+                best, pick = cost, (bd, k)
+            k += 1
+        bd //= 2
+    return pick
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_the_cheapest_of_all_cuts(cut, shape):
+    rng = random.Random(77)
+    for _ in range(150):
+        n, chunk = int(2 ** rng.uniform(1, 17)), int(2 ** rng.uniform(13, 34))
+        s = cut(chunk, n, shape)
+        if s["align"]:  # else the CTA may be smaller than the cut's
+            assert (s["threads"], s["parts"]) == _every_cut(chunk, n, shape), (chunk, n)
+
+
+@pytest.mark.parametrize("chunk,n,shape", [(100000, 153, SHAPES[0]), (1 << 20, 7, SHAPES[2]), (77474, 64, SHAPES[-1])])
+def test_host_time(cut, chunk, n, shape):
+    """Short reduces: the cut costs the host less than 120 divisions (each cut tried by
+    itself took 220 to 540, this takes 20 to 40)."""
+    assert cut(chunk, n, shape, divisions=True) < 120
