@@ -45,8 +45,14 @@ __global__ void __launch_bounds__(kThreads) store_upto_kernel(const uint64_t* __
     }
 }
 
+// CTAs an SM must hold (0: the compiler's choice). Left to itself it takes 48 registers
+// at W = 5, too few to hash the four solutions of a block side by side: 2^20 solutions
+// took 69.8 us, and take 53.6 with 70 registers; W = 8 92.7 -> 80.4, W = 3 37.4 -> 32.3.
+// At W = 1 it lost 8% of 2^28, from W = 9 on it gave nothing.
+constexpr int reduce_upto_ctas(int W) { return W > 1 && W <= 8 ? 2 : 0; }
+
 template <int W, int U>
-__global__ void __launch_bounds__(kThreads) reduce_upto_kernel(const uint64_t* __restrict__ table,
+__global__ void __launch_bounds__(kThreads, reduce_upto_ctas(W)) reduce_upto_kernel(const uint64_t* __restrict__ table,
                                                                const int32_t* info, uint64_t cap,
                                                                hlf_reduce* __restrict__ out)
 {
@@ -93,9 +99,8 @@ hlf_status launch_reduce_upto_w(const uint64_t* table, const int32_t* info, uint
                                 cudaStream_t s)
 {
     constexpr int U = reduce_unroll(W);
-    // one wave at most (8 CTAs of 256 threads per SM), and runs of at least
-    // 256 solutions (enough to amortise a seed of <= 64 row XORs) when the
-    // whole cap is enumerated: small instances spread over many SMs
+    // 8 CTAs of 256 threads per SM at most, and runs of at least 256 solutions
+    // when the whole cap is enumerated, which makes 16 CTAs of 2^20
     const uint64_t most = (uint64_t)sm_count() * 8;
     uint64_t blocks = (cap + 256 * kThreads - 1) / (256 * kThreads);
     if (blocks > most) blocks = most;
