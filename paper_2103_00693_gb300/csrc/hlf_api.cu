@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "hlf_internal.cuh"
+#include "slots.h"
 #include "upto.cuh"
 
 struct hlf_handle {
@@ -156,12 +157,11 @@ cudaStream_t release_stream(int dev)
     return streams[dev];
 }
 
-// Per device, made on first need and kept until the process exits: a stream and
-// pinned memory for hlf_get_factor's copies, used by one call at a time. With a stream
-// of the handle's own and a copy of each array to pageable memory, stage 1 of n = 1024
-// with its results on the host took 205 us; with one copy through here 162.
+// Made on first need and kept until the process exits: a stream and pinned memory for
+// hlf_get_factor's copies, used by one call at a time. With a stream of the handle's own
+// and a copy of each array to pageable memory, stage 1 of n = 1024 with its results on
+// the host took 205 us; with one copy through here 162.
 struct CopyBuffer {
-    std::mutex mu;
     cudaStream_t stream = nullptr;
     unsigned char* pinned = nullptr;
 };
@@ -181,11 +181,21 @@ hlf_status ensure_copy_buffer(CopyBuffer& c)
     return HLF_OK;
 }
 
-CopyBuffer* copy_buffer(int dev)
+// A device's: as many threads copy side by side, further ones wait for one of them.
+using CopyBuffers = hlf::Slots<CopyBuffer, 8>;
+CopyBuffers* copy_buffers(int dev)
 {
-    static CopyBuffer buffers[64];
+    static CopyBuffers buffers[64];
     return dev < 0 || dev >= 64 ? nullptr : &buffers[dev];
 }
+
+// One of them for the length of a call.
+struct CopyTurn {
+    CopyBuffers& all;
+    CopyBuffer* c;
+    explicit CopyTurn(CopyBuffers& a) : all(a), c(a.take()) {}
+    ~CopyTurn() { all.give(c); }
+};
 
 // Host wait for every stream's latest work through h.
 hlf_status wait_uses(hlf_handle* h)
@@ -485,15 +495,16 @@ hlf_status hlf_get_factor(hlf_handle* h, int32_t* piv_host, uint64_t* z0_host, u
     hlf_status st = ensure_rank(h);
     if (st != HLF_OK) return st;
     const size_t W = h->W, r = h->r;
-    CopyBuffer* c = copy_buffer(h->device);
-    if (!c) return HLF_ERR_CUDA;
+    CopyBuffers* buffers = copy_buffers(h->device);
+    if (!buffers) return HLF_ERR_CUDA;
     // the pivots, tables and basis rows are one block (see hlf_factor)
     const unsigned char* from = reinterpret_cast<const unsigned char*>(h->piv);
     const size_t at_z0 = reinterpret_cast<const unsigned char*>(h->table + hlf::kTableZ0Row * W) - from;
     const size_t at_basis = reinterpret_cast<const unsigned char*>(h->basis) - from;
     const size_t bytes = basis_host ? at_basis + sizeof(uint64_t) * W * r : at_z0 + sizeof(uint64_t) * W;
     if (bytes > kCopyBytes) return HLF_ERR_INTERNAL;
-    std::lock_guard<std::mutex> lock(c->mu);
+    CopyTurn turn(*buffers);
+    CopyBuffer* c = turn.c;
     st = ensure_copy_buffer(*c);
     if (st != HLF_OK) return st;
     if (cudaMemcpyAsync(c->pinned, from, bytes, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
