@@ -121,6 +121,7 @@ __global__ void clear_results_kernel(uint64_t* __restrict__ out, uint64_t words)
 // inside gave 2%; the hash's last shift or its sum on the multiply pipe lost 1-10%.
 
 constexpr int kRegionMin = 33;
+static_assert(kRegionMin > 32, "a region's basis has a row of zero low word");
 
 // x = (lo, hi) behind the second shift: the last product and shift, added to hs.
 __device__ __forceinline__ void region_tail(uint32_t lo, uint32_t hi, uint64_t& hs)
@@ -259,11 +260,11 @@ __global__ void __launch_bounds__(1024, 1) reduce_region_kernel(const uint64_t* 
         cnt = min(per, size - j);
         uint64_t z[1];
         seed_lookup<1>(st, ntab, j, z);
+        // u >= m - 32 >= 1: at most 32 of the m rows are pivots on the 32-bit low word
         if (u >= 4) region_run<4>(t, j, cnt, z[0], acc.hs);
         else if (u == 3) region_run<3>(t, j, cnt, z[0], acc.hs);
         else if (u == 2) region_run<2>(t, j, cnt, z[0], acc.hs);
-        else if (u == 1) region_run<1>(t, j, cnt, z[0], acc.hs);
-        else reduce_run_from<1, kRegionBlock>(t, false, j, cnt, z, acc);
+        else region_run<1>(t, j, cnt, z[0], acc.hs);
     }
     block_reduce<1, 1024>(cnt, acc);
     if (threadIdx.x == 0 && cnt) {
