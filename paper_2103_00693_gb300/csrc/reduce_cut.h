@@ -88,17 +88,25 @@ inline ReduceShape reduce_shape(uint64_t chunk, uint64_t n_chunks, int U, uint64
     }
     const uint64_t slots = sms * fit(sh.threads), items = n_chunks * sh.parts;
     sh.blocks = (unsigned)(items < slots ? items : slots);
-    // A window with too few Gray blocks for the threads at hand, a CTA's if all windows
-    // run at once, else those of a warp, is dealt to them by the index: idle lanes cost
-    // as much as walking ones. With a Gray block a thread instead, 10^5 windows of 10 at
-    // W = 11 took 1207 us (now 421), 20000 of 100 at W = 2 129 (47), 152 of 10 at W = 16
-    // 13.4 (8.3); dealt over all 1024 threads of a CTA, 64 of 5000 at W = 4 12.4 (8.3).
-    const uint64_t lanes = items > slots ? 32 : (sh.threads < kFew ? sh.threads : kFew);
-    if (sh.parts == 1 && chunk <= lanes * ((1ull << U) - 1)) {
-        if (items <= slots) sh.threads = (unsigned)lanes;
-        sh.per = (chunk + lanes - 1) / lanes;
-        sh.runs = (chunk + sh.per - 1) / sh.per;
-        return sh;
+    if (sh.parts == 1) {
+        // Where all windows run at once a CTA needs no more threads than its window has
+        // Gray blocks: 100 of 2000 at W = 4 6.5 us with 256, 8.4 with 1024.
+        const bool at_once = items <= slots;
+        const uint64_t use = runs < kFew ? kFew : (runs + 31) / 32 * 32;
+        if (at_once && use < sh.threads) sh.threads = (unsigned)use;
+        // A window with too few blocks for the threads at hand, a CTA's if all windows run
+        // at once, else those of a warp, is dealt to them by the index: idle lanes cost
+        // as much as walking ones. With a block a thread instead, 10^5 windows of 10 at
+        // W = 11 took 1207 us (now 421), 20000 of 100 at W = 2 129 (47), 152 of 10 at W = 16
+        // 13.4 (8.3). Lanes that would walk more than about a third of a block do no better
+        // so: 608 of 300 at W = 11, three a lane, 14.5 us, in blocks of four 12.3.
+        const uint64_t lanes = !at_once ? 32 : (sh.threads < kFew ? sh.threads : kFew);
+        if (chunk <= lanes * (at_once ? ((1ull << U) + 2) / 3 : (1ull << U) - 1)) {
+            if (at_once) sh.threads = (unsigned)lanes;
+            sh.per = (chunk + lanes - 1) / lanes;
+            sh.runs = (chunk + sh.per - 1) / sh.per;
+            return sh;
+        }
     }
     want = (uint64_t)sh.parts * sh.threads;
     // chunk + 2^U - 1 indices at most, counted from the window's first block;

@@ -51,7 +51,8 @@ def test_unroll_change(made):
 
 
 @pytest.mark.parametrize("n", [40, 250, 1000])
-@pytest.mark.parametrize("chunk,n_chunks", [(1, 3000), (2, 153), (9, 1), (63, 40), (8193, 3), (50001, 153), (70000, 7)])
+@pytest.mark.parametrize("chunk,n_chunks", [(1, 3000), (2, 153), (9, 1), (63, 40), (8193, 3), (50001, 153), (70000, 7),
+                                           (10, 5000), (96, 2000), (97, 2000), (300, 400), (512, 9), (513, 9), (769, 9), (2001, 100)])
 def test_chunks(made, n, chunk, n_chunks):
     F, G = made[n]
     off = 3

@@ -108,7 +108,22 @@ def test_short_windows_fill_lanes(cut, shape):
     U = shape[1]
     for chunk in (2, 10, 31, 32 * ((1 << U) - 1)):
         assert cut(chunk, 100000, shape)["per"] <= (chunk + 31) // 32
+    for chunk in (2, 10, 100, 256 * (((1 << U) + 2) // 3)):
         assert cut(chunk, 7, shape)["per"] <= (chunk + 255) // 256
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_cta_no_larger_than_its_window(cut, shape):
+    """Windows that all run at once: 256 threads, or one for each Gray block; lanes walk
+    whole blocks where they would have more than a third of a block each."""
+    U = shape[1]
+    for chunk in (300, 2000):
+        for n in (7, 100, 400):
+            s = cut(chunk, n, shape)
+            if s["parts"] > 1 or n > SMS * _fit(shape, s["threads"]):
+                continue
+            assert s["threads"] <= max(256, ((chunk - 1 >> U) + 2 + 31) // 32 * 32)
+            assert s["align"] or s["per"] <= ((1 << U) + 2) // 3
 
 
 @pytest.mark.parametrize("shape", SHAPES)
@@ -140,8 +155,10 @@ def test_the_cheapest_of_all_cuts(cut, shape):
     for _ in range(150):
         n, chunk = int(2 ** rng.uniform(1, 17)), int(2 ** rng.uniform(13, 34))
         s = cut(chunk, n, shape)
-        if s["align"]:  # else the CTA may be smaller than the cut's
-            assert (s["threads"], s["parts"]) == _every_cut(chunk, n, shape), (chunk, n)
+        threads, parts = _every_cut(chunk, n, shape)
+        assert s["parts"] == parts, (chunk, n)
+        if parts > 1 or n > SMS * _fit(shape, threads):  # else the CTA may be smaller than the cut's
+            assert s["threads"] == threads, (chunk, n)
 
 
 @pytest.mark.parametrize("chunk,n,shape", [(100000, 153, SHAPES[0]), (1 << 20, 7, SHAPES[2]), (77474, 64, SHAPES[-1])])
