@@ -19,14 +19,15 @@
 //                        per CTA. One window or many (a result per chunk).
 //                        Windows too short to give a full wave long runs are
 //                        bound by how many threads walk them: runs go down
-//                        to one Gray block.
+//                        to one Gray block, and below that to single indices
+//                        (reduce_cut.h).
 //   store_kernel         coalesced materialisation by groups of 64 or 32
 //                        consecutive solutions a warp step (store_groups): one
 //                        XOR per solution, 512 B a step at W = 1; at W > 1 the
 //                        lanes' solutions are restaged in shared memory so that
 //                        the warp writes its 32*W words with consecutive lanes
 //                        on consecutive words. Bound by HBM stores.
-//   sample_kernel        z(i) at arbitrary indices, straight from the formula.
+//   sample_kernel        z(i) at arbitrary indices, by lookups in seed tables.
 
 #include "enum_impl.cuh"
 #include "reduce_cut.h"

@@ -2,7 +2,7 @@
 // r from the words the factor kernel left in the handle's device memory.
 //   store_upto_kernel   stores z(i) = z0 ^ XOR_{k in g(i)} B_k (Eq. 3 with
 //                       the Gray-code basis order) for every i < min(2^r, cap),
-//                       each straight from the definition. Meant for
+//                       each by lookups in seed tables. Meant for
 //                       instances of up to a few million solutions, where the
 //                       time is the launch and the host round trip it saves;
 //                       hlf_enumerate_store walks large windows.

@@ -49,7 +49,8 @@ def test_histogram_argument_checks(cuda_ok):
 
 def _first_rows_independent(F, lo, nb, rows):
     """Whether the field bits [lo, lo + nb) of the enumeration rows 0..4 are
-    linearly independent over GF(2) (the kernel then walks lane-interleaved)."""
+    linearly independent over GF(2) (every aligned block of 32 solutions then
+    counts 32 bins once)."""
     vecs = [int(sum(int(b) << j for j, b in enumerate(r[lo:lo + nb]))) for r in rows[:5]]
     if len(vecs) < 5:
         return False
@@ -66,8 +67,8 @@ def _first_rows_independent(F, lo, nb, rows):
 @pytest.mark.parametrize("order", ["gray", "paper"])
 def test_histogram_both_walks(cuda_ok, order):
     """Fields whose bits over the first five enumeration rows are independent
-    (the lane-interleaved walk) and fields where they are not (per-thread
-    runs), each against the oracle over windows with ragged ends."""
+    (small blocks spread over their bins) and fields where they are not (they
+    count one bin often), each against the oracle over windows with ragged ends."""
     A = synth.grid_instance(7, 0.5, 21)
     F = oc.factor(A)
     G = hlf.Factorization.from_dense(A)
@@ -84,13 +85,13 @@ def test_histogram_both_walks(cuda_ok, order):
             cnt = min(cnt, space - off)
             got = G.histogram(off, cnt, lo, nb).cpu().numpy().view(np.uint64)
             assert np.array_equal(got, oc.histogram(F, off, cnt, lo, nb, order)), (order, lo, nb, off, cnt)
-    assert seen == {True, False}, "both walks should be exercised"
+    assert seen == {True, False}, "both kinds of field should be exercised"
     G.close()
 
 
 def test_histogram_window_ending_at_2_64(cuda_ok):
     """r > 64: the index space is [0, 2^64), and a window may end exactly at
-    2^64 (the end wraps to 0 in 64-bit arithmetic); both walks."""
+    2^64 (the end wraps to 0 in 64-bit arithmetic)."""
     A = synth.random_symmetric(100, 0.02, 140)
     F = oc.factor(A)
     assert F.r > 64
@@ -104,8 +105,8 @@ def test_histogram_window_ending_at_2_64(cuda_ok):
 
 
 def test_atomic_probe_counts_every_atomic(cuda_ok):
-    """The shared-memory atomic microbenchmark behind the histogram's
-    roofline performs exactly the atomics it reports."""
+    """The shared-memory atomic microbenchmark performs exactly the atomics it
+    reports."""
     import torch
 
     s = torch.empty(1, dtype=torch.int64, device="cuda")
